@@ -33,6 +33,7 @@
 #include <string>
 
 #include "../../include/lbm.h"
+#include "lbm_widesum.cuh"
 
 void lbm_internal_set_global_error(const std::string& msg);  // lbm_api.cu
 
@@ -87,19 +88,30 @@ __global__ void __launch_bounds__(kThreads) k_partials(const float* __restrict__
     const size_t N = (size_t)n_nodes;
     for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < n_nodes; n += gridDim.x * blockDim.x) {
         if (flags && (flags[n] == kFlagSolid || flags[n] == kFlagSymmetry)) continue;
-        bool bad = false;
-        for (int a = 0; a < 27; ++a) {
-            const float x = f[a * N + n];
-            bad |= !isfinite(x);
-            v[0] += (double)x;
-        }
-        for (int i = 0; i < qh; ++i) {
-            const float x = h[i * N + n];
-            bad |= !isfinite(x);
-            v[1] += (double)x;
+        // a node's values as wide sums (the FP64 pipe would bound the kernel), the nodes in FP64
+        lbmd::WideSum<float> sumf, sumh;
+#pragma unroll
+        for (int a = 0; a < 27; ++a) sumf.add(f[a * N + n]);
+#pragma unroll 7
+        for (int i = 0; i < qh; ++i) sumh.add(h[i * N + n]);
+        if (isfinite(sumf.hi) && isfinite(sumh.hi)) {
+            v[0] += sumf.value();
+            v[1] += sumh.value();
+        } else {  // a non-finite value, or a sum beyond the float range: one by one in FP64
+            bool bad = false;
+            for (int a = 0; a < 27; ++a) {
+                const float x = f[a * N + n];
+                bad |= !isfinite(x);
+                v[0] += (double)x;
+            }
+            for (int i = 0; i < qh; ++i) {
+                const float x = h[i * N + n];
+                bad |= !isfinite(x);
+                v[1] += (double)x;
+            }
+            v[2] += bad ? 1.0 : 0.0;
         }
         if (theta) v[1] -= 0.5 * (double)theta[n];
-        v[2] += bad ? 1.0 : 0.0;
         v[3] += 1.0;
     }
     warp_block_sum(v, sh);

@@ -1,0 +1,59 @@
+"""The FP64 totals and wall sums of the library against exactly rounded sums
+(math.fsum) of the populations that it stores, at sizes around the edges of
+their kernels: a few nodes, more nodes than one sweep of the grid, ragged ones.
+
+Tolerance of the totals: a node's values are added as an FP32 pair (error 2^-48
+of the node's sum of magnitudes per addition, 53 additions), nodes in FP64
+(2^-53 of the running total per addition): 2^-42 of the sum of all magnitudes
+bounds both."""
+import math
+
+import numpy as np
+import pytest
+
+from paper_2203_01316_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+def _box(dims, storage, qh):
+    from paper_2203_01316_gb300 import Solver
+    nx, ny, nz = dims
+    N = nx * ny * nz
+    s = Solver(nx, ny, nz, nu=0.02, k=1e-3, lat_h=qh, storage=storage, periodic_x=True, T_ref=0.3)
+    s.set_geometry(np.zeros(N, np.uint8))
+    s.init_fields(1.0 + I.uniform(1, N, -1e-2, 1e-2), I.uniform(2, 3 * N, -0.05, 0.05), I.uniform(3, N, 0.0, 1.0))
+    return s, N
+
+
+def _stored(s, N, qh, storage):
+    """The stored deviations as float64 [27 + qh, N]."""
+    import torch
+    buf = s.save_state(torch.empty(s.state_size(), dtype=torch.uint8, device="cuda"))
+    dt = {"f32": torch.float32, "f64": torch.float64, "f16": torch.float16, "bf16": torch.bfloat16}[storage]
+    size = torch.empty(0, dtype=dt).element_size()
+    return buf, buf[-(27 + qh) * N * size:].view(dt).view(27 + qh, N)
+
+
+@pytest.mark.parametrize("qh", [27, 7])
+@pytest.mark.parametrize("storage", ["f32", "f64", "f16", "bf16"])
+@pytest.mark.parametrize("dims", [(1, 1, 1), (33, 7, 5), (101, 67, 53)])
+def test_totals_equal_the_exact_sums(dims, storage, qh):
+    s, N = _box(dims, storage, qh)
+    v = _stored(s, N, qh, storage)[1].double().cpu().numpy()
+    mass, energy = s.balances()
+    for got, x, shift in ((mass, v[:27], 1.0 * N), (energy, v[27:], 0.3 * N)):
+        assert abs(got - (math.fsum(x.reshape(-1)) + shift)) <= 2.0 ** -42 * (np.abs(x).sum() + shift)
+
+
+@pytest.mark.parametrize("qh", [27, 7])
+def test_totals_of_values_beyond_the_float_range(qh):
+    """Finite values whose sum is no float: the FP64 total is finite, the state is not diverged."""
+    s, N = _box((9, 5, 3), "f32", qh)
+    buf, v = _stored(s, N, qh, "f32")
+    v[3, 17] = v[5, 17] = 3e38
+    s.load_state(buf)
+    mass, energy = s.balances()
+    x = v.double().cpu().numpy()
+    assert mass == pytest.approx(math.fsum(x[:27].reshape(-1)) + N, rel=1e-12)
+    assert energy == pytest.approx(math.fsum(x[27:].reshape(-1)) + 0.3 * N, rel=1e-12)
