@@ -52,7 +52,7 @@ struct lbm_ctx {
     std::vector<float> Twall{0.0f};
     float* d_theta = nullptr;
     void* d_inlet = nullptr;  // R[27 + qh]
-    double* d_scratch = nullptr;  // 3 * kRedBlocks partials + 4 results
+    double* d_scratch = nullptr;  // 3 * kRedBlocks partials + 4 results + the counter of the reductions
     double* d_stage = nullptr;    // 5 * N doubles for host-side outputs
     int64_t n_fluid_like = 0;     // non-solid node count
     bool geometry = false, initialised = false;
@@ -352,13 +352,14 @@ lbm_status lbm_create(const lbm_params* params, lbm_ctx** out) {
     }
     if (dev_alloc(c, &c->d_flags, N) != cudaSuccess ||
         dev_alloc(c, &c->d_inlet, (27 + 27) * sizeof(double)) != cudaSuccess ||
-        dev_alloc(c, &c->d_scratch, (3 * lbmd::kRedBlocks + 4) * sizeof(double)) != cudaSuccess ||
+        dev_alloc(c, &c->d_scratch, (3 * lbmd::kRedBlocks + 5) * sizeof(double)) != cudaSuccess ||
         dev_alloc(c, &c->d_Twall, sizeof(float)) != cudaSuccess)
         return bail(fail(c, LBM_ERR_NOMEM, "context buffers: out of device memory"));
     if (c->ssize == 2 && dev_alloc(c, &c->d_stepctr, sizeof(uint32_t)) != cudaSuccess)
         return bail(fail(c, LBM_ERR_NOMEM, "step counter: out of device memory"));
 
     cudaMemsetAsync(c->d_flags, 0, N, c->stream);
+    cudaMemsetAsync(c->d_scratch, 0, (3 * lbmd::kRedBlocks + 5) * sizeof(double), c->stream);
     cudaMemsetAsync(c->d_Twall, 0, sizeof(float), c->stream);
 
     DevParams& d = c->dp;

@@ -763,6 +763,109 @@ cudaError_t launch_balances(const Buffers& b, const DevParams& p, double* scratc
     return cudaGetLastError();
 }
 
+// ---- wall sums: one lane per link ---------------------------------------------
+// A group of lanes takes one wall node, lane i its direction i, so that the
+// links of a node load together; a thread that walked its node's links one
+// after another waited for each link's loads in turn (384x128x128 sphere: flux
+// 34 us, force 44 us and two reductions of 5 us; fields, totals, flux and force
+// of that state 764 -> 711 us).  Each lane keeps one direction throughout, so the links' values
+// are added as a WideSum and multiplied by the lane's constants once at the end.
+constexpr int kWallLanes27 = 32, kWallLanes7 = 8;
+template <int QH> constexpr int wall_lanes() { return QH == 27 ? kWallLanes27 : kWallLanes7; }
+
+// direction of a run-time index (the tables above packed into constants)
+__host__ __device__ constexpr uint64_t pack_e(int d) {
+    uint64_t v = 0;
+    for (int a = 0; a < 27; ++a) v |= (uint64_t)((d == 0 ? EX(a) : (d == 1 ? EY(a) : EZ(a))) + 1) << (2 * a);
+    return v;
+}
+struct LaneDir {
+    int a, b;           // D3Q27 index and its opposite
+    int ex, ey, ez;
+    double w;           // D3Q27 weight
+};
+__device__ __forceinline__ LaneDir lane_dir(int a) {
+    constexpr uint64_t px = pack_e(0), py = pack_e(1), pz = pack_e(2);
+    LaneDir l;
+    l.a = a;
+    l.ex = (int)(px >> (2 * a) & 3) - 1;
+    l.ey = (int)(py >> (2 * a) & 3) - 1;
+    l.ez = (int)(pz >> (2 * a) & 3) - 1;
+    int b = 0;
+#pragma unroll
+    for (int k = 1; k < 27; ++k)
+        if (k == a) b = OPP(k);
+    l.b = b;
+    const int zeros = (l.ex == 0) + (l.ey == 0) + (l.ez == 0);
+    l.w = (double)(1 << (2 * zeros)) / 216.0;  // 4^zeros / 216
+    return l;
+}
+// node x - e_a of a wall node: its x_f, the source of population a
+__device__ __forceinline__ int lane_src(const LaneDir& l, int x, int y, int z, const DevParams& p) {
+    int xs = x - l.ex, ys = y - l.ey, zs = z - l.ez;
+    if (p.periodic_x) xs = xs < 0 ? xs + p.nx : (xs >= p.nx ? xs - p.nx : xs);
+    else xs = min(max(xs, 0), p.nx - 1);
+    ys = ys < 0 ? ys + p.ny : (ys >= p.ny ? ys - p.ny : ys);
+    zs = zs < 0 ? zs + p.nz : (zs >= p.nz ? zs - p.nz : zs);
+    return xs + p.nx * (ys + p.ny * zs);
+}
+// blocks of a wall sum: every lane group of a block takes a few nodes
+inline int wall_blocks(int nw, int lanes) {
+    const int64_t b = ((int64_t)nw * lanes + kRedThreads - 1) / kRedThreads;
+    return (int)std::min<int64_t>(std::max<int64_t>(b, 1), kRedBlocks);
+}
+
+// The last block of a reduction to arrive adds the blocks' partial sums (in
+// block order, so the result does not depend on which block that is); true in
+// its thread 0, with the totals in v.  ctr: a counter that is zero before and
+// after (atomicInc wraps it).
+template <int NV>
+__device__ __forceinline__ bool reduce_in_last_block(double (&v)[NV], double* sh, double* __restrict__ part,
+                                                     unsigned* __restrict__ ctr) {
+    __shared__ bool last;
+    block_sum<NV>(v, sh);
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) part[blockIdx.x * NV + k] = v[k];
+        __threadfence();
+        last = atomicInc(ctr, gridDim.x - 1) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = 0.0;
+    for (int i = threadIdx.x; i < gridDim.x; i += blockDim.x)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) v[k] += __ldcg(part + i * NV + k);
+    __syncthreads();  // sh is free again
+    block_sum<NV>(v, sh);
+    return threadIdx.x == 0;
+}
+
+// what a reduction does with its totals: out[k] = v[k], or (acc given)
+// *acc += weight * v[pick]
+struct RedOut {
+    double* out;
+    double* acc;
+    double weight;
+    int pick;
+};
+template <int NV> __device__ __forceinline__ void write_totals(const double (&v)[NV], const RedOut& o) {
+    if (o.acc) {
+        double x = v[0];
+#pragma unroll
+        for (int k = 1; k < NV; ++k)
+            if (o.pick == k) x = v[k];
+        *o.acc += o.weight * x;
+    } else {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) o.out[k] = v[k];
+    }
+}
+// the counter of reduce_in_last_block lies behind the partials and results
+__host__ __device__ inline unsigned* red_counter(double* scratch) { return (unsigned*)(scratch + 3 * kRedBlocks + 4); }
+
 // surface heat flux of one wall (Sec. 4.4): for every IABB link of the wall,
 // h_ibar(x_b, t+1) from Eq. IABB minus h*_i(x_b, t); the shifts cancel
 template <typename S, int QH>
@@ -773,56 +876,60 @@ __global__ void __launch_bounds__(kRedThreads) k_surface_flux(const S* __restric
                                                               const float* __restrict__ lq,
                                                               const int32_t* __restrict__ lwall,
                                                               const float* __restrict__ Twall, int nw, int wall,
-                                                              double* __restrict__ part, const DevParams p) {
+                                                              double* __restrict__ part, const RedOut o,
+                                                              const DevParams p) {
     using R = typename Acc<S>::R;
+    constexpr int L = wall_lanes<QH>();
     __shared__ double sh[32];
-    double v[1] = {0.0};
     const size_t N = (size_t)p.N;
     const R Tref = par<R>(p.Tref, p.pf.Tref);
-    for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < nw; w += gridDim.x * blockDim.x) {
-        const int n = wnode[w];
+    const int ia = threadIdx.x % L;  // h population of this lane
+    const LaneDir d = lane_dir(QH == 27 ? min(ia, 26) : (ia < 4 ? ia : min(ia + 3, 9)));
+    const int ib = QH == 27 ? d.b : OPP7(min(ia, 6));
+    const R wi = QH == 27 ? (R)d.w : (R)(1.0 / 6.0);
+    const R heq2 = R(2) * wi * ((R)Twall[wall] - Tref);
+    WideSum<R> sum;
+    const int step = gridDim.x * (blockDim.x / L);
+    for (int w = blockIdx.x * (blockDim.x / L) + threadIdx.x / L; w < nw; w += step) {
         const uint32_t mask = wmask[w];
-        const int off = woff[w];
-        int x, y, z;
-        node_xyz(n, p, x, y, z);
-        const Nbr nb = make_nbr(x, y, z, p);
-#pragma unroll
-        for (int ia = 0; ia < QH; ++ia) {
-            const int a = HDIR<QH>(ia);
-            if (!(mask & (1u << a))) continue;
-            const int l = off + __popc(mask & ((1u << a) - 1u));
-            if (lwall[l] != wall) continue;
-            const int ib = HOPP<QH>(ia);
-            const int b = HDIR<QH>(ib);
-            const float q = lq[l];
-            const R heq2 = R(2) * (R)HW<QH>(ia) * ((R)Twall[wall] - Tref);
-            const bool thin = (mask >> b) & 1u;
-            const R ha_b = ld<R>(hA + ia * N + n);
-            R hin;
-            if (p.wall_bc == 1) {
-                hin = R(0.5) * heq2;
-            } else if (q <= 0.5f && !thin) {
-                const R ha_f = ld<R>(hA + ia * N + src_of(nb, a));
-                hin = -(R(2) * (R)q * ha_b + (R(1) - R(2) * (R)q) * ha_f) + heq2;
-            } else {
-                const R qq = (R)fmaxf(q, 0.5f);
-                const R hb_b = ld<R>(hA + ib * N + n);
-                hin = (-ha_b + (R(2) * qq - R(1)) * hb_b + heq2) / (R(2) * qq);
-            }
-            v[0] += (double)hin - (double)ha_b;
+        if (ia == 0 || ia >= QH || !(mask >> d.a & 1u)) continue;
+        const int l = woff[w] + __popc(mask & ((1u << d.a) - 1u));
+        if (lwall[l] != wall) continue;
+        const int n = wnode[w];
+        const float q = lq[l];
+        const bool thin = (mask >> d.b) & 1u;
+        const R ha_b = ld<R>(hA + ia * N + n);
+        R hin;
+        if (p.wall_bc == 1) {
+            hin = R(0.5) * heq2;
+        } else if (q <= 0.5f && !thin) {
+            int x, y, z;
+            node_xyz(n, p, x, y, z);
+            const R ha_f = ld<R>(hA + ia * N + lane_src(d, x, y, z, p));
+            hin = -(R(2) * (R)q * ha_b + (R(1) - R(2) * (R)q) * ha_f) + heq2;
+        } else {
+            const R qq = (R)fmaxf(q, 0.5f);
+            const R hb_b = ld<R>(hA + ib * N + n);
+            hin = (-ha_b + (R(2) * qq - R(1)) * hb_b + heq2) / (R(2) * qq);
         }
+        sum.add(hin);
+        sum.add(-ha_b);
     }
-    block_sum<1>(v, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = v[0];
+    double v[1] = {sum.value()};
+    if (reduce_in_last_block<1>(v, sh, part, red_counter(part))) write_totals<1>(v, o);
 }
 
 template <typename S, int QH>
+cudaError_t surface_flux_to(const Buffers& b, const DevParams& p, int wall, double* scratch, const RedOut& o,
+                            cudaStream_t s) {
+    k_surface_flux<S, QH><<<wall_blocks(b.nw, wall_lanes<QH>()), kRedThreads, 0, s>>>(
+        (const S*)b.hA, b.wnode, b.wmask, b.woff, b.lq, b.lwall, b.Twall, b.nw, wall, scratch, o, p);
+    return cudaGetLastError();
+}
+template <typename S, int QH>
 cudaError_t launch_surface_flux(const Buffers& b, const DevParams& p, int wall, double* scratch, double* out,
                                 cudaStream_t s) {
-    k_surface_flux<S, QH><<<kRedBlocks, kRedThreads, 0, s>>>((const S*)b.hA, b.wnode, b.wmask, b.woff, b.lq, b.lwall,
-                                                            b.Twall, b.nw, wall, scratch, p);
-    k_reduce_partials<1><<<1, 1024, 0, s>>>(scratch, kRedBlocks, out);
-    return cudaGetLastError();
+    return surface_flux_to<S, QH>(b, p, wall, scratch, RedOut{out, nullptr, 0.0, 0}, s);
 }
 
 // force on one wall by momentum exchange (Ladd 1994, Mei et al. 2002; not in
@@ -836,55 +943,55 @@ __global__ void __launch_bounds__(kRedThreads) k_wall_force(const S* __restrict_
                                                             const int32_t* __restrict__ woff,
                                                             const float* __restrict__ lq,
                                                             const int32_t* __restrict__ lwall, int nw, int wall,
-                                                            double* __restrict__ part, const DevParams p) {
+                                                            double* __restrict__ part, const RedOut o,
+                                                            const DevParams p) {
     using R = typename Acc<S>::R;
+    constexpr int L = kWallLanes27;
     __shared__ double sh[3 * 32];
-    double v[3] = {0.0, 0.0, 0.0};
     const size_t N = (size_t)p.N;
-    for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < nw; w += gridDim.x * blockDim.x) {
-        const int n = wnode[w];
+    const int ia = threadIdx.x % L;
+    const LaneDir d = lane_dir(min(ia, 26));
+    WideSum<R> sum;
+    int links = 0;
+    const int step = gridDim.x * (blockDim.x / L);
+    for (int w = blockIdx.x * (blockDim.x / L) + threadIdx.x / L; w < nw; w += step) {
         const uint32_t mask = wmask[w];
-        const int off = woff[w];
-        int x, y, z;
-        node_xyz(n, p, x, y, z);
-        const Nbr nb = make_nbr(x, y, z, p);
-#pragma unroll
-        for (int a = 1; a < 27; ++a) {
-            if (!(mask & (1u << a))) continue;
-            const int l = off + __popc(mask & ((1u << a) - 1u));
-            if (lwall[l] != wall) continue;
-            const int b = OPP(a);
-            const float q = lq[l];
-            const bool thin = (mask >> b) & 1u;  // x_f = x_b - e_a is solid
-            const R fa_b = ld<R>(fA + a * N + n);
-            R fin;
-            if (q <= 0.5f && !thin) {
-                fin = R(2) * (R)q * fa_b + (R(1) - R(2) * (R)q) * ld<R>(fA + a * N + src_of(nb, a));
-            } else {
-                const R qq = (R)fmaxf(q, 0.5f);
-                fin = (fa_b + (R(2) * qq - R(1)) * ld<R>(fA + b * N + n)) / (R(2) * qq);
-            }
-            const double carried = (double)fa_b + (double)fin + 2.0 * W27(a) * p.rho0;
-            v[0] += EX(a) * carried;
-            v[1] += EY(a) * carried;
-            v[2] += EZ(a) * carried;
+        if (ia == 0 || ia >= 27 || !(mask >> d.a & 1u)) continue;
+        const int l = woff[w] + __popc(mask & ((1u << d.a) - 1u));
+        if (lwall[l] != wall) continue;
+        const int n = wnode[w];
+        const float q = lq[l];
+        const bool thin = (mask >> d.b) & 1u;  // x_f = x_b - e_a is solid
+        const R fa_b = ld<R>(fA + d.a * N + n);
+        R fin;
+        if (q <= 0.5f && !thin) {
+            int x, y, z;
+            node_xyz(n, p, x, y, z);
+            fin = R(2) * (R)q * fa_b + (R(1) - R(2) * (R)q) * ld<R>(fA + d.a * N + lane_src(d, x, y, z, p));
+        } else {
+            const R qq = (R)fmaxf(q, 0.5f);
+            fin = (fa_b + (R(2) * qq - R(1)) * ld<R>(fA + d.b * N + n)) / (R(2) * qq);
         }
+        sum.add(fa_b);
+        sum.add(fin);
+        ++links;
     }
-    block_sum<3>(v, sh);
-    if (threadIdx.x == 0) {
-        part[3 * blockIdx.x] = v[0];
-        part[3 * blockIdx.x + 1] = v[1];
-        part[3 * blockIdx.x + 2] = v[2];
-    }
+    const double carried = sum.value() + 2.0 * d.w * p.rho0 * (double)links;
+    double v[3] = {d.ex * carried, d.ey * carried, d.ez * carried};
+    if (reduce_in_last_block<3>(v, sh, part, red_counter(part))) write_totals<3>(v, o);
 }
 
+template <typename S>
+cudaError_t wall_force_to(const Buffers& b, const DevParams& p, int wall, double* scratch, const RedOut& o,
+                          cudaStream_t s) {
+    k_wall_force<S><<<wall_blocks(b.nw, kWallLanes27), kRedThreads, 0, s>>>(
+        (const S*)b.fA, b.wnode, b.wmask, b.woff, b.lq, b.lwall, b.nw, wall, scratch, o, p);
+    return cudaGetLastError();
+}
 template <typename S, int QH>
 cudaError_t launch_wall_force(const Buffers& b, const DevParams& p, int wall, double* scratch, double* out,
                               cudaStream_t s) {
-    k_wall_force<S><<<kRedBlocks, kRedThreads, 0, s>>>((const S*)b.fA, b.wnode, b.wmask, b.woff, b.lq, b.lwall,
-                                                      b.nw, wall, scratch, p);
-    k_reduce_partials<3><<<1, 1024, 0, s>>>(scratch, kRedBlocks, out);
-    return cudaGetLastError();
+    return wall_force_to<S>(b, p, wall, scratch, RedOut{out, nullptr, 0.0, 0}, s);
 }
 
 // ---- adjoint of the h evolution --------------------------------------------
@@ -2300,26 +2407,13 @@ cudaError_t launch_record_h(const Buffers& b, const DevParams& p, void* rec, cud
     return cudaGetLastError();
 }
 
-template <int NV>
-__global__ void k_reduce_accumulate(const double* __restrict__ part, int nparts, int pick, double weight,
-                                    double* __restrict__ acc) {
-    __shared__ double sh[32 * NV];
-    double v[NV];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) v[k] = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x)
-#pragma unroll
-        for (int k = 0; k < NV; ++k) v[k] += part[i * NV + k];
-    block_sum<NV>(v, sh);
-    if (threadIdx.x == 0) acc[0] += weight * v[pick];
-}
-
 // x-flux sum e_x h through the plane x = plane (Sec. 4.4 section flux; the
 // shift w T_ref carries no x-flux)
 template <typename S, int QH>
 __global__ void __launch_bounds__(kRedThreads) k_section_flux(const S* __restrict__ hA,
                                                               const uint8_t* __restrict__ flags, int plane,
-                                                              double* __restrict__ part, const DevParams p) {
+                                                              double* __restrict__ part, const RedOut o,
+                                                              const DevParams p) {
     using R = typename Acc<S>::R;
     __shared__ double sh[32];
     double v[1] = {0.0};
@@ -2334,25 +2428,18 @@ __global__ void __launch_bounds__(kRedThreads) k_section_flux(const S* __restric
             if (ex != 0) v[0] += (double)ex * (double)ld<R>(hA + i * N + n);
         }
     }
-    block_sum<1>(v, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = v[0];
+    if (reduce_in_last_block<1>(v, sh, part, red_counter(part))) write_totals<1>(v, o);
 }
 
 template <typename S, int QH>
 cudaError_t launch_objective(const Buffers& b, const DevParams& p, AdjObjective obj, double* scratch, double* acc,
                              cudaStream_t s) {
-    if (obj.kind == 2) {
-        k_wall_force<S><<<kRedBlocks, kRedThreads, 0, s>>>((const S*)b.fA, b.wnode, b.wmask, b.woff, b.lq, b.lwall,
-                                                          b.nw, obj.wall, scratch, p);
-        k_reduce_accumulate<3><<<1, 1024, 0, s>>>(scratch, kRedBlocks, obj.comp, obj.weight, acc);
-        return cudaGetLastError();
-    }
-    if (obj.kind == 0)
-        k_surface_flux<S, QH><<<kRedBlocks, kRedThreads, 0, s>>>((const S*)b.hA, b.wnode, b.wmask, b.woff, b.lq,
-                                                                b.lwall, b.Twall, b.nw, obj.wall, scratch, p);
-    else
-        k_section_flux<S, QH><<<kRedBlocks, kRedThreads, 0, s>>>((const S*)b.hA, b.flags, obj.plane, scratch, p);
-    k_reduce_accumulate<1><<<1, 1024, 0, s>>>(scratch, kRedBlocks, 0, obj.weight, acc);
+    const RedOut o{nullptr, acc, obj.weight, obj.kind == 2 ? obj.comp : 0};
+    if (obj.kind == 2) return wall_force_to<S>(b, p, obj.wall, scratch, o, s);
+    if (obj.kind == 0) return surface_flux_to<S, QH>(b, p, obj.wall, scratch, o, s);
+    const int rows = p.ny * p.nz;
+    k_section_flux<S, QH><<<std::min((rows + kRedThreads - 1) / kRedThreads, kRedBlocks), kRedThreads, 0, s>>>(
+        (const S*)b.hA, b.flags, obj.plane, scratch, o, p);
     return cudaGetLastError();
 }
 

@@ -57,3 +57,32 @@ def test_totals_of_values_beyond_the_float_range(qh):
     x = v.double().cpu().numpy()
     assert mass == pytest.approx(math.fsum(x[:27].reshape(-1)) + N, rel=1e-12)
     assert energy == pytest.approx(math.fsum(x[27:].reshape(-1)) + 0.3 * N, rel=1e-12)
+
+
+@pytest.mark.parametrize("qh", [27, 7])
+@pytest.mark.parametrize("wall_bc", ["iabb", "eq"])
+@pytest.mark.parametrize("dims", [(6, 5, 3), (70, 9, 41), (300, 5, 131)])
+def test_wall_sums_of_one_and_of_many_sweeps(dims, wall_bc, qh):
+    """Surface flux and force of two walls between which the links alternate, against the oracle; the last grid
+    has more wall nodes (78,600) than one sweep of the reduction's lane groups (9,728 or 38,912)."""
+    from oracle import oracle as O
+    from paper_2203_01316_gb300 import Solver
+    nx, ny, nz = dims
+    N = nx * ny * nz
+    flags = I.channel_flags(nx, ny, nz, periodic_x=True)
+    links = I.plate_walls(flags, 0.3, 0.8)
+    links["wall"] = (np.arange(len(links["node"])) % 2).astype(np.int32)
+    rho, u, T = 1.0 + I.uniform(1, N, -1e-2, 1e-2), I.uniform(2, 3 * N, -0.05, 0.05), I.uniform(3, N, 0.0, 1.0)
+    s = Solver(nx, ny, nz, nu=0.02, k=1e-3, lat_h=qh, storage="f64", periodic_x=True, T_ref=0.3, wall_bc=wall_bc)
+    o = O.Oracle(O.make_params(nx=nx, ny=ny, nz=nz, qh=qh, periodic_x=True, nu=0.02, k=1e-3, wall_bc=wall_bc))
+    s.set_geometry(flags.reshape(-1), links, n_walls=2)
+    o.set_geometry(flags, links, nwalls=2)
+    for w, Tw in enumerate((0.25, 1.5)):
+        s.set_bc(w, Tw)
+        o.set_wall_temperature(w, Tw)
+    s.init_fields(rho, u, T)
+    o.init_fields(rho, u, T)
+    tol = 1e-13 * len(links["node"])  # FP64 link values of O(1), each within a few hundred ulp of the oracle's
+    for w in range(2):
+        assert abs(s.surface_flux(w) - o.surface_flux(w)) <= tol
+        assert np.abs(s.wall_force(w) - o.wall_force(w)).max() <= tol
