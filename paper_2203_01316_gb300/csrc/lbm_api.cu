@@ -42,7 +42,7 @@ struct lbm_ctx {
     int32_t* d_roff = nullptr;
     int32_t* d_rlink = nullptr;
     double* d_dlink = nullptr;      // adjoint: per link dJ/dT_w accumulators
-    double* d_flowacc = nullptr;    // coupled adjoint: per node (dJ/dF, dJ/du_in) accumulators, [N][6]
+    double* d_flowacc = nullptr;    // coupled adjoint: dJ/dF per warp and dJ/du_in per inlet row
     void* d_din = nullptr;          // coupled adjoint: d(inlet state)/du_in, R[3][27 + qh]
     void* d_wflow = nullptr;        // coupled adjoint: velocity derivative of the h step, R[3][N]
     uint32_t* d_stepctr = nullptr;  // 16-bit storage: the time level replayed step graphs read
@@ -1375,6 +1375,10 @@ lbm_status lbm_step_record_pre(lbm_ctx* c, int n, void* f_rec, void* h_rec) {
     return LBM_OK;
 }
 
+static size_t flow_acc_bytes(const lbm_ctx* c) {
+    return 3 * (lbmd::flow_acc_warps(c->N) + (size_t)c->p.ny * c->p.nz) * sizeof(double);
+}
+
 lbm_status lbm_adjoint_flow_step(lbm_ctx* c, const void* f_level, const void* h_level, const void* muf_next,
                                  const void* muh_next, void* muf_out, void* muh_out, const lbm_objective* obj,
                                  double* dJ_dtheta) {
@@ -1389,9 +1393,9 @@ lbm_status lbm_adjoint_flow_step(lbm_ctx* c, const void* f_level, const void* h_
     DeviceGuard g(c->device);
     const size_t rsize = c->ssize;
     if (!c->d_flowacc) {
-        if (dev_alloc(c, &c->d_flowacc, (size_t)c->N * 6 * sizeof(double)) != cudaSuccess)
+        if (dev_alloc(c, &c->d_flowacc, flow_acc_bytes(c)) != cudaSuccess)
             return fail(c, LBM_ERR_NOMEM, "coupled adjoint accumulators: out of device memory");
-        CK(cudaMemsetAsync(c->d_flowacc, 0, (size_t)c->N * 6 * sizeof(double), c->stream), "accumulators");
+        CK(cudaMemsetAsync(c->d_flowacc, 0, flow_acc_bytes(c), c->stream), "accumulators");
     }
     if (!c->d_din && dev_alloc(c, &c->d_din, (size_t)3 * (27 + c->qh) * rsize) != cudaSuccess)
         return fail(c, LBM_ERR_NOMEM, "inlet derivative table: out of device memory");
@@ -1444,16 +1448,16 @@ lbm_status lbm_adjoint_flow_gradient(lbm_ctx* c, double* dJ_dF, double* dJ_duin,
     DeviceGuard g(c->device);
     for (int d = 0; d < 3; ++d) dJ_dF[d] = dJ_duin[d] = 0.0;
     if (!c->d_flowacc) return LBM_OK;
-    CK(lbmd::launch_reduce6(c->d_flowacc, c->N, c->d_scratch, c->stream), "flow gradient reduction");
-    double out[6];
-    CK(cudaMemcpyAsync(out, c->d_scratch, sizeof(out), cudaMemcpyDeviceToHost, c->stream), "flow gradient copy");
-    if (reset)
-        CK(cudaMemsetAsync(c->d_flowacc, 0, (size_t)c->N * 6 * sizeof(double), c->stream), "flow gradient reset");
+    double* out = c->d_scratch + 3 * lbmd::kRedBlocks;  // three results, read back before the next use
+    const size_t nw = lbmd::flow_acc_warps(c->N);
+    CK(lbmd::launch_reduce3(c->d_flowacc, (int)nw, c->p.storage == LBM_F32, out, c->d_scratch, c->stream),
+       "flow gradient reduction");
+    CK(cudaMemcpyAsync(dJ_dF, out, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "flow gradient copy");
+    CK(lbmd::launch_reduce3(c->d_flowacc + 3 * nw, c->p.ny * c->p.nz, false, out, c->d_scratch, c->stream),
+       "flow gradient reduction");
+    CK(cudaMemcpyAsync(dJ_duin, out, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "flow gradient copy");
+    if (reset) CK(cudaMemsetAsync(c->d_flowacc, 0, flow_acc_bytes(c), c->stream), "flow gradient reset");
     CK(cudaStreamSynchronize(c->stream), "flow gradient");
-    for (int d = 0; d < 3; ++d) {
-        dJ_dF[d] = out[d];
-        dJ_duin[d] = out[3 + d];
-    }
     return LBM_OK;
 }
 

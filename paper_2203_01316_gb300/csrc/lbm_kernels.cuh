@@ -50,6 +50,10 @@ struct AdjObjective {
 };
 
 constexpr int kBlock = 128;
+// warps of the coupled sweep; its accumulators are [warps][3] for dJ/dF
+// (WideSum, 8 bytes each for either arithmetic), then FP64 [ny nz][3] for dJ/du_in
+inline size_t flow_acc_warps(int N) { return (size_t)((N + kBlock - 1) / kBlock) * (kBlock / 32); }
+static_assert(sizeof(WideSum<float>) == 8 && sizeof(WideSum<double>) == 8, "one slot size");
 constexpr int kRedBlocks = 1216;  // 8 x 152 SMs, partial sums of the reductions
 constexpr int kRedThreads = 256;
 
@@ -68,16 +72,16 @@ cudaError_t launch_inlet(const Buffers& b, const DevParams& p, cudaStream_t s, b
 // symmetry rows: fill them in the post-collision arrays before a step
 template <typename S, int QH>
 cudaError_t launch_mirror(const Buffers& b, const DevParams& p, cudaStream_t s);
-// out[0..5] = sum over the n nodes of acc[n * 6 + k] (the coupled adjoint's
-// per-node dJ/dF, dJ/du_in accumulators)
-cudaError_t launch_reduce6(const double* acc, int n, double* out, cudaStream_t s);
+// out[k] = sum of acc[i * 3 + k] over i < n (the coupled adjoint's accumulators);
+// pairs: acc holds WideSum<float>
+cudaError_t launch_reduce3(const double* acc, int n, bool pairs, double* out, double* scratch, cudaStream_t s);
 // adjoint of one level of the coupled f + h evolution (records of the level's
 // pre-collision arrivals; f_level NULL at the initial level); wbuf: R[3][N]
 // scratch for the velocity derivative passed from the h to the f kernel
 template <typename R, int QH>
 cudaError_t launch_adjoint_flow(const Buffers& b, const DevParams& p, const R* f_level, const R* h_level,
                                 const R* muf_next, const R* muh_next, R* muf_out, R* muh_out, AdjObjective obj,
-                                double* dtheta, double* acc6, const R* din, R* wbuf, cudaStream_t s);
+                                double* dtheta, double* acc, const R* din, R* wbuf, cudaStream_t s);
 // rec[i * N + n] = post-collision h deviation of population i at node n (type R)
 template <typename S, int QH>
 cudaError_t launch_record_h(const Buffers& b, const DevParams& p, void* rec, cudaStream_t s);
@@ -1053,7 +1057,7 @@ template <typename R> __device__ __forceinline__ void z_from_lambda27(R* cb, R u
 }
 template <typename R>
 __device__ __forceinline__ void transpose_from_z27(R* cb, R ux, R uy, R uz, const DevParams& p, R* mu,
-                                                   double& dth) {
+                                                   WideSum<R>& dth) {
     R rank = R(0);
 #pragma unroll
     for (int o = 0; o < 3; ++o)
@@ -1065,7 +1069,7 @@ __device__ __forceinline__ void transpose_from_z27(R* cb, R ux, R uy, R uz, cons
                 const R sr = par<R>(p.sh[m + nn + o], p.pf.sh[m + nn + o]);
                 R& v = cb[MIDX(m, nn, o)];
                 if (E != R(0)) {
-                    dth += (double)(E * v);
+                    dth.add(E * v);
                     rank += E * sr * v;
                 }
                 v *= (R(1) - sr);
@@ -1090,8 +1094,7 @@ __device__ __forceinline__ void transpose_from_z27(R* cb, R ux, R uy, R uz, cons
 template <typename R, int QH, bool CUM>
 __device__ __forceinline__ void h_collision_transpose(const R* lam, const R* hpost, const R ux, const R uy,
                                                       const R uz, const R Q, const DevParams& p, R* mu,
-                                                      double& dth) {
-    dth = 0.0;
+                                                      WideSum<R>& dth) {
     if constexpr (CUM) {
         // Cumulants-1st (Eq. H_cu_collision): s^k = (H + Q) M(v), M the unit
         // equilibrium at v = (1 - s) m + s u, m = sum e g / H, H = sum g of the
@@ -1160,7 +1163,7 @@ __device__ __forceinline__ void h_collision_transpose(const R* lam, const R* hpo
             const int a = HDIR<QH>(i);
             mu[i] = base + c1 * (EX(a) * G[0] + EY(a) * G[1] + EZ(a) * G[2]);
         }
-        dth = (double)L0;
+        dth.add(L0);
     } else if constexpr (QH == 27) {
         R cb[27];
 #pragma unroll
@@ -1182,7 +1185,8 @@ __device__ __forceinline__ void h_collision_transpose(const R* lam, const R* hpo
             z0 += u[d] * mb1 + u[d] * u[d] * mb2;
         }
         const R s0 = par<R>(p.sh[0], p.pf.sh[0]), s1 = par<R>(p.sh[1], p.pf.sh[1]), s2 = par<R>(p.sh[2], p.pf.sh[2]);
-        dth = (double)z0 + (double)(c * (z2[0] + z2[1] + z2[2]));
+        dth.add(z0);
+        dth.add(c * (z2[0] + z2[1] + z2[2]));
         const R rank = s0 * z0 + s2 * c * (z2[0] + z2[1] + z2[2]);
         z0 *= (R(1) - s0);
 #pragma unroll
@@ -1352,7 +1356,7 @@ __global__ void __launch_bounds__(kBlock) k_adjoint(const R* __restrict__ mu_nex
         return;
     }
     const R ux = uk[n], uy = uk[N + n], uz = uk[2 * N + n];
-    double dth = 0.0;
+    WideSum<R> dth;
     {
         R mu[QH], hp[QH];
         if constexpr (CUM) {
@@ -1365,7 +1369,7 @@ __global__ void __launch_bounds__(kBlock) k_adjoint(const R* __restrict__ mu_nex
 #pragma unroll
         for (int i = 0; i < QH; ++i) out[soa(i, N, n)] = mu[i];
     }
-    if (dtheta) dtheta[n] += dth;
+    if (dtheta) dtheta[n] += dth.value();
 }
 
 template <typename R, int QH>
@@ -1796,14 +1800,13 @@ __device__ __forceinline__ void h_velocity_adjoint(const R* lam, const R* g, R u
 // functions)
 template <typename R, int QH>
 __device__ __forceinline__ void h_transpose_and_velocity(const R* lam, const R* g, R ux, R uy, R uz, R Q,
-                                                         const DevParams& p, R* mu, double& dth, R* w) {
+                                                         const DevParams& p, R* mu, WideSum<R>& dth, R* w) {
     if constexpr (QH == 27) {
         R Z[27];
 #pragma unroll
         for (int a = 0; a < 27; ++a) Z[CUBE(a)] = lam[a];
         z_from_lambda27<R>(Z, ux, uy, uz);
         velocity_from_z27<R>(Z, g, ux, uy, uz, Q, p, w);
-        dth = 0.0;
         transpose_from_z27<R>(Z, ux, uy, uz, p, mu, dth);
     } else {
         h_velocity_adjoint<R, QH>(lam, g, ux, uy, uz, Q, p, w);
@@ -2074,15 +2077,18 @@ __device__ __forceinline__ void flow_velocity(const R* m, const DevParams& p, R&
 // written to wbuf[3][N], dJ/dQ, the wall-temperature terms); PART 2, the f
 // adjoint (gather of mu_f, the reversed f collision with w, dJ/dF).  PART 1
 // runs first.
+// dF receives the node's (dC_f/dF)^T lambda_f + (dU/dF)^T w (PART 2; zeros
+// where the node has none).
 template <typename R, int QH, bool CUM, int PART>
-__global__ void __launch_bounds__(kBlock) k_adjoint_flow(
+__device__ __forceinline__ void adjoint_flow_node(
     const R* __restrict__ muf_next, const R* __restrict__ muh_next, R* __restrict__ muf_out, R* __restrict__ muh_out,
     const R* __restrict__ gf, const R* __restrict__ gh, const float* __restrict__ theta,
-    double* __restrict__ dtheta, double* __restrict__ acc6, const R* __restrict__ din, R* __restrict__ wbuf,
+    double* __restrict__ dtheta, double* __restrict__ acc_in, const R* __restrict__ din, R* __restrict__ wbuf,
     const uint8_t* __restrict__ flags, const int32_t* __restrict__ seg_base, const uint32_t* __restrict__ wmask,
     const int32_t* __restrict__ woff, const float* __restrict__ lq, const int32_t* __restrict__ lwall,
     const int32_t* __restrict__ rseg_base, const uint32_t* __restrict__ rmask, const int32_t* __restrict__ roff,
-    const int32_t* __restrict__ rlink, double* __restrict__ dlink, const AdjObjective obj, const DevParams p) {
+    const int32_t* __restrict__ rlink, double* __restrict__ dlink, const AdjObjective& obj, const DevParams& p,
+    R (&dF)[3]) {
     using D = Dual<R>;
     constexpr bool HP = PART == 1, FP = PART == 2;
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2257,7 +2263,7 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_flow(
 #pragma unroll
                 for (int i = 0; i < QH; ++i) acc += (double)(din[d * (27 + QH) + 27 + i] * lh[i]);
             }
-            acc6[(size_t)n * 6 + 3 + d] += acc;
+            acc_in[(size_t)(n / p.nx) * 3 + d] += acc;  // x = 0: row y + ny z
         }
         if constexpr (FP) {
 #pragma unroll
@@ -2301,7 +2307,7 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_flow(
         // mu_h = (dC_h/dg_h)^T lambda_h and dJ/dQ, transposed exactly (the
         // h-only adjoint's code; Cumulants-1st needs the post-collision
         // state); the central-moment kinds get w from the same z
-        double dth = 0.0;
+        WideSum<R> dth;
         R muh[QH];
         if constexpr (CUM) {
             R hp[QH];
@@ -2319,18 +2325,65 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_flow(
         // here; k_zou_he_adjoint then transposes the rule that built it)
 #pragma unroll
         for (int i = 0; i < QH; ++i) muh_out[i * N + n] = muh[i];
-        if (dtheta) dtheta[n] += dth;
+        if (dtheta) dtheta[n] += dth.value();
     } else {
         const R w[3] = {wbuf[n], wbuf[N + n], wbuf[2 * N + n]};
         // G_k for the ten unit-moment perturbations (k < 10) and the force (10..12)
         R G[13];
         collide_f_adjoint<R>(g, p, lf, w, G);
 #pragma unroll
-        for (int d = 0; d < 3; ++d) acc6[(size_t)n * 6 + d] += (double)G[10 + d];
+        for (int d = 0; d < 3; ++d) dF[d] = G[10 + d];
         R mf[27];
         moments_transpose_f<R>(G, mf);
 #pragma unroll
         for (int b = 0; b < 27; ++b) muf_out[b * N + n] = mf[b];
+    }
+}
+
+// accF[warp][3]: accumulators of dJ/dF as WideSum (a warp adds its nodes' terms
+// of a level there), acc_in[row][3]: FP64 accumulators of dJ/du_in per inlet
+// row.  Each slot has one owner, so there are no atomics.  One FP64 slot of six
+// per node took 96 B of the f part's 460 B per node, six operations a node on
+// the FP64 pipe, and 1.4 ms to add up at 192x64x64 (60 levels and their
+// recomputation there: 26.30 -> 22.36 ms, with dJ/dQ as WideSum, which took the
+// h part from 102 to 93 us)
+template <typename R, int QH, bool CUM, int PART>
+__global__ void __launch_bounds__(kBlock) k_adjoint_flow(
+    const R* __restrict__ muf_next, const R* __restrict__ muh_next, R* __restrict__ muf_out, R* __restrict__ muh_out,
+    const R* __restrict__ gf, const R* __restrict__ gh, const float* __restrict__ theta,
+    double* __restrict__ dtheta, WideSum<R>* __restrict__ accF, double* __restrict__ acc_in, const R* __restrict__ din,
+    R* __restrict__ wbuf, const uint8_t* __restrict__ flags, const int32_t* __restrict__ seg_base,
+    const uint32_t* __restrict__ wmask, const int32_t* __restrict__ woff, const float* __restrict__ lq,
+    const int32_t* __restrict__ lwall, const int32_t* __restrict__ rseg_base, const uint32_t* __restrict__ rmask,
+    const int32_t* __restrict__ roff, const int32_t* __restrict__ rlink, double* __restrict__ dlink,
+    const AdjObjective obj, const DevParams p) {
+    R dF[3] = {R(0), R(0), R(0)};
+    adjoint_flow_node<R, QH, CUM, PART>(muf_next, muh_next, muf_out, muh_out, gf, gh, theta, dtheta, acc_in, din, wbuf,
+                                        flags, seg_base, wmask, woff, lq, lwall, rseg_base, rmask, roff, rlink, dlink,
+                                        obj, p, dF);
+    if constexpr (PART == 2) {
+        if (!gf) return;
+        // through shared memory eight lanes take a component, four nodes each:
+        // 60 instructions a thread where shuffles alone take 160
+        __shared__ R sh[kBlock / 32][3][40];  // 40: the components on different banks
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, d = lane >> 3, i = lane & 7;
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 3; ++k) sh[warp][k][lane] = dF[k];
+        __syncwarp();
+        WideSum<R> v;
+        if (d < 3) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v.add(sh[warp][d][i + 8 * k]);
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) v.merge_down(o);
+        if (d < 3 && i == 0) {
+            WideSum<R>* slot = accF + (size_t)((blockIdx.x * kBlock + threadIdx.x) >> 5) * 3 + d;
+            WideSum<R> t = *slot;
+            t.merge(v);
+            *slot = t;
+        }
     }
 }
 
@@ -2341,7 +2394,7 @@ template <typename R, int QH>
 __global__ void __launch_bounds__(kBlock) k_zou_he_adjoint(R* __restrict__ muf, R* __restrict__ muh,
                                                             const R* __restrict__ gf, const R* __restrict__ gh,
                                                             const uint8_t* __restrict__ flags,
-                                                            double* __restrict__ acc6, const DevParams p) {
+                                                            double* __restrict__ acc_in, const DevParams p) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= p.ny * p.nz) return;
     const int n = p.nx * i;  // x = 0, row i = y + ny z
@@ -2359,7 +2412,7 @@ __global__ void __launch_bounds__(kBlock) k_zou_he_adjoint(R* __restrict__ muf, 
         h[k] = gh[k * N + n];
         mh[k] = muh[k * N + n];
     }
-    zou_he_transpose_coupled<R, QH>(g, h, mf, mh, p, acc6 + (size_t)n * 6 + 3);
+    zou_he_transpose_coupled<R, QH>(g, h, mf, mh, p, acc_in + (size_t)i * 3);
 #pragma unroll
     for (int a = 0; a < 27; ++a) muf[a * N + n] = mf[a];
 #pragma unroll
@@ -2369,10 +2422,12 @@ __global__ void __launch_bounds__(kBlock) k_zou_he_adjoint(R* __restrict__ muf, 
 template <typename R, int QH>
 cudaError_t launch_adjoint_flow(const Buffers& b, const DevParams& p, const R* f_level, const R* h_level,
                                 const R* muf_next, const R* muh_next, R* muf_out, R* muh_out, AdjObjective obj,
-                                double* dtheta, double* acc6, const R* din, R* wbuf, cudaStream_t s) {
+                                double* dtheta, double* acc, const R* din, R* wbuf, cudaStream_t s) {
     const int grid = (p.N + kBlock - 1) / kBlock;
+    WideSum<R>* accF = (WideSum<R>*)acc;
+    double* acc_in = acc + 3 * flow_acc_warps(p.N);
 #define LBM_ADJF_ARGS                                                                                            \
-    muf_next, muh_next, muf_out, muh_out, f_level, h_level, b.theta, dtheta, acc6, din, wbuf, b.flags,          \
+    muf_next, muh_next, muf_out, muh_out, f_level, h_level, b.theta, dtheta, accF, acc_in, din, wbuf, b.flags,  \
         b.seg_base, b.wmask, b.woff, b.lq, b.lwall, b.rseg_base, b.rmask, b.roff, b.rlink, b.dlink, obj, p
     if (p.hkind == 3) {
         k_adjoint_flow<R, QH, true, 1><<<grid, kBlock, 0, s>>>(LBM_ADJF_ARGS);
@@ -2385,7 +2440,7 @@ cudaError_t launch_adjoint_flow(const Buffers& b, const DevParams& p, const R* f
     if (p.zou_he && f_level) {
         const int rows = p.ny * p.nz;
         k_zou_he_adjoint<R, QH><<<(rows + kBlock - 1) / kBlock, kBlock, 0, s>>>(muf_out, muh_out, f_level, h_level,
-                                                                              b.flags, acc6, p);
+                                                                              b.flags, acc_in, p);
     }
     return cudaGetLastError();
 }

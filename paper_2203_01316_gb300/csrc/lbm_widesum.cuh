@@ -16,6 +16,9 @@ namespace lbmd {
 template <typename R> struct WideSum {
     R hi = R(0);
     __device__ __forceinline__ void add(R x) { hi += x; }
+    __device__ __forceinline__ void merge(const WideSum& v) { hi += v.hi; }
+    // adds the sum of the lane o lanes up
+    __device__ __forceinline__ void merge_down(int o) { hi += __shfl_down_sync(0xffffffffu, hi, o); }
     __device__ __forceinline__ double value() const { return (double)hi; }
 };
 template <> struct WideSum<float> {
@@ -25,6 +28,16 @@ template <> struct WideSum<float> {
         const float b = __fadd_rn(s, -hi);  // the part of x that s holds
         lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -b)), __fadd_rn(x, -b)));
         hi = s;
+    }
+    __device__ __forceinline__ void merge(const WideSum& v) {
+        add(v.hi);
+        lo = __fadd_rn(lo, v.lo);
+    }
+    __device__ __forceinline__ void merge_down(int o) {
+        WideSum v;
+        v.hi = __shfl_down_sync(0xffffffffu, hi, o);
+        v.lo = __shfl_down_sync(0xffffffffu, lo, o);
+        merge(v);
     }
     __device__ __forceinline__ double value() const {
         return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
