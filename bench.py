@@ -127,7 +127,8 @@ def kernel_source_hash(csrc=None):
     parts = [dev,
              _between(ker, "constexpr int kBlock", "\n"),
              _between(ker, "#ifdef LBM_KERNEL_TU", "template <typename S, int QH>\ncudaError_t launch_step("),
-             _between(ker, "cudaError_t launch_step(const Buffers& b, const DevParams& p, cudaStream_t s, bool advance_h) {",
+             _between(ker, "cudaError_t launch_step(const Buffers& b, const DevParams& p, cudaStream_t s, bool advance_h, "
+                      "cudaStream_t walls) {",
                       "\n}\n")]
     h = hashlib.sha256()
     for t in parts:

@@ -75,6 +75,10 @@ struct lbm_ctx {
     } graphs[2];
     int graph_next = 0;
     bool graph_broken = false;  // capture failed once: plain launches from then on
+    // second branch of captured steps: the wall nodes' launch and the Zou-He
+    // inlet, which write other nodes than the step's own launch
+    cudaStream_t side = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
 };
 
 static std::string g_create_err;
@@ -421,6 +425,9 @@ lbm_status lbm_destroy(lbm_ctx* c) {
     cudaFree(c->d_stepctr);
     for (auto& gr : c->graphs)
         if (gr.exec) cudaGraphExecDestroy(gr.exec);
+    if (c->fork) cudaEventDestroy(c->fork);
+    if (c->join) cudaEventDestroy(c->join);
+    if (c->side) cudaStreamDestroy(c->side);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
     return LBM_OK;
@@ -851,55 +858,89 @@ lbm_status lbm_init_fields(lbm_ctx* c, const double* rho, const double* u, const
     return LBM_OK;
 }
 
-// the Zou-He inlet plane, after each step
-static cudaError_t zou_he_inlet(lbm_ctx* c, const Buffers& b, const DevParams& p, bool advance_h) {
+// the Zou-He inlet plane of a step, on stream s
+static cudaError_t zou_he_inlet(lbm_ctx* c, const Buffers& b, const DevParams& p, bool advance_h, cudaStream_t s) {
     if (!p.zou_he) return cudaSuccess;
     return dispatch(c, [&](auto tag) {
         using Tg = decltype(tag);
-        return lbmd::launch_inlet<typename Tg::S, Tg::Q>(b, p, c->stream, advance_h);
+        return lbmd::launch_inlet<typename Tg::S, Tg::Q>(b, p, s, advance_h);
     });
 }
 
-// symmetry rows take their mirrored populations before each step
-static cudaError_t fill_mirror(lbm_ctx* c, const Buffers& b, const DevParams& p) {
+// symmetry rows of the current level
+static cudaError_t fill_mirror(lbm_ctx* c, const Buffers& b) {
+    const DevParams& p = c->dp;
     if (!p.mirror_lo && !p.mirror_hi) return cudaSuccess;
     return dispatch(c, [&](auto tag) {
         using Tg = decltype(tag);
         return lbmd::launch_mirror<typename Tg::S, Tg::Q>(b, p, c->stream);
     });
 }
+// before the first step of a call (the state may come from lbm_init_fields or
+// lbm_load_state) where the steps then keep the rows; launch_level fills them
+// for each step otherwise
+static lbm_status fill_mirror_once(lbm_ctx* c) {
+    if (!lbmd::step_fills_symmetry(c->ssize, c->qh)) return LBM_OK;
+    const cudaError_t e = fill_mirror(c, buffers(c));
+    return e == cudaSuccess ? LBM_OK : cuda_fail(c, e, "symmetry rows launch");
+}
 
-// the launches of one plain step (symmetry rows, the step, the Zou-He inlet)
+// the launches of one step: the step's own and the Zou-He inlet.  forked (in
+// a graph capture): the inlet and the wall nodes' launch go to the side branch
+static cudaError_t launch_level(lbm_ctx* c, const Buffers& b, const DevParams& p, bool advance_h, bool forked = false) {
+    cudaError_t e = lbmd::step_fills_symmetry(c->ssize, c->qh) ? cudaSuccess : fill_mirror(c, b);
+    if (e != cudaSuccess) return e;
+    const cudaStream_t side = forked ? c->side : c->stream;
+    if (forked) {
+        if ((e = cudaEventRecord(c->fork, c->stream)) != cudaSuccess) return e;
+        if ((e = cudaStreamWaitEvent(side, c->fork, 0)) != cudaSuccess) return e;
+        if ((e = zou_he_inlet(c, b, p, advance_h, side)) != cudaSuccess) return e;
+    }
+    e = dispatch(c, [&](auto tag) {
+        using Tg = decltype(tag);
+        return lbmd::launch_step<typename Tg::S, Tg::Q>(b, p, c->stream, advance_h, side);
+    });
+    if (e != cudaSuccess) return e;
+    if (!forked) return zou_he_inlet(c, b, p, advance_h, side);
+    if ((e = cudaEventRecord(c->join, side)) != cudaSuccess) return e;
+    return cudaStreamWaitEvent(c->stream, c->join, 0);
+}
+
 // the time-level counter of replayed 16-bit step graphs: set before a run
-// of replays, advanced inside each captured step
+// of replays, advanced at the end of each captured pair of steps
 __global__ void k_step_counter(uint32_t* ctr, uint32_t value, int advance) {
-    if (advance) *ctr += 1u;
+    if (advance) *ctr += value;
     else *ctr = value;
 }
 
-// one plain step; in_graph: the step is being captured for replay, so with
-// stochastically rounded 16-bit storage its kernels read the time level from
-// the device counter, which the step advances first
-static lbm_status step_once(lbm_ctx* c, bool in_graph = false) {
+// one plain step; level > 0: it is being captured for replay as the level-th
+// step of its graph, so with 16-bit storage its kernels take the time level
+// from the device counter (which the graph advances at its end) plus level
+static lbm_status step_once(lbm_ctx* c, int level = 0, bool forked = false) {
     const Buffers b = buffers(c);
     c->dp.step += 1;
     DevParams p = c->dp;
-    cudaError_t e;
-    if (in_graph && c->d_stepctr) {
-        k_step_counter<<<1, 1, 0, c->stream>>>(c->d_stepctr, 0u, 1);
-        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "step counter launch");
+    if (level > 0 && c->d_stepctr) {
         p.step_ctr = c->d_stepctr;
+        p.step = (uint32_t)level;
     }
-    if ((e = fill_mirror(c, b, p)) != cudaSuccess) return cuda_fail(c, e, "symmetry rows launch");
-    e = dispatch(c, [&](auto tag) {
-        using Tg = decltype(tag);
-        return lbmd::launch_step<typename Tg::S, Tg::Q>(b, p, c->stream);
-    });
+    const cudaError_t e = launch_level(c, b, p, true, forked);
     if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
-    if ((e = zou_he_inlet(c, b, p, true)) != cudaSuccess) return cuda_fail(c, e, "inlet launch");
     c->cur_f = 1 - c->cur_f;
     c->cur_h = 1 - c->cur_h;
     return LBM_OK;
+}
+
+// whether captured steps have a side branch (its stream and events made at
+// first use; without them the launches stay in one line)
+static bool side_branch(lbm_ctx* c) {
+    if (!c->dp.zou_he && !(c->ssize == 2 && c->dp.nwall > 0)) return false;
+    if (!c->side && cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess) c->side = nullptr;
+    if (!c->fork && cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess) c->fork = nullptr;
+    if (!c->join && cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming) != cudaSuccess) c->join = nullptr;
+    if (c->side && c->fork && c->join) return true;
+    cudaGetLastError();
+    return false;
 }
 
 // A graph of two plain steps for the current buffers and parameters
@@ -927,10 +968,15 @@ static lbm_ctx::StepGraph* step_graph(lbm_ctx* c) {
     const std::string err = c->err;
     cudaGraph_t graph = nullptr;
     lbm_status st = LBM_OK;
+    const bool forked = side_branch(c);
     cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        st = step_once(c, true);
-        if (st == LBM_OK) st = step_once(c, true);
+        st = step_once(c, 1, forked);
+        if (st == LBM_OK) st = step_once(c, 2, forked);
+        if (st == LBM_OK && c->d_stepctr) {
+            k_step_counter<<<1, 1, 0, c->stream>>>(c->d_stepctr, 2u, 1);
+            if (cudaGetLastError() != cudaSuccess) st = LBM_ERR_CUDA;
+        }
         e = cudaStreamEndCapture(c->stream, &graph);
     }
     // the captured launches did not run: undo their bookkeeping
@@ -959,6 +1005,10 @@ lbm_status lbm_step(lbm_ctx* c, int n) {
     if (n < 0) return fail(c, LBM_ERR_INVALID, "n must be >= 0");
     if (!c->initialised) return fail(c, LBM_ERR_STATE, "initialise the fields first");
     DeviceGuard g(c->device);
+    if (n > 0) {
+        const lbm_status st = fill_mirror_once(c);
+        if (st != LBM_OK) return st;
+    }
     // launch-bound stretches replay graphs of two steps (LBM_STEP_AUTO)
     const bool graphs = c->p.step_kernel == LBM_STEP_AUTO && !c->graph_broken && n >= 4;
     if (graphs) {
@@ -1254,19 +1304,15 @@ lbm_status lbm_step_record(lbm_ctx* c, int n, void* u_rec, int advance_h) {
     if (!c->initialised) return fail(c, LBM_ERR_STATE, "initialise the fields first");
     DeviceGuard g(c->device);
     const size_t rsize = c->p.storage == LBM_F64 ? sizeof(double) : sizeof(float);
+    lbm_status st = n > 0 ? fill_mirror_once(c) : LBM_OK;
+    if (st != LBM_OK) return st;
     for (int i = 0; i < n; ++i) {
         Buffers b = buffers(c);
         c->dp.step += 1;
         const DevParams p = c->dp;
         b.urec = (char*)u_rec + (size_t)i * 3 * c->N * rsize;
-        cudaError_t e = fill_mirror(c, b, p);
-        if (e != cudaSuccess) return cuda_fail(c, e, "symmetry rows launch");
-        e = dispatch(c, [&](auto tag) {
-            using Tg = decltype(tag);
-            return lbmd::launch_step<typename Tg::S, Tg::Q>(b, p, c->stream, advance_h != 0);
-        });
+        const cudaError_t e = launch_level(c, b, p, advance_h != 0);
         if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
-        if ((e = zou_he_inlet(c, b, p, advance_h != 0)) != cudaSuccess) return cuda_fail(c, e, "inlet launch");
         c->cur_f = 1 - c->cur_f;
         if (advance_h) c->cur_h = 1 - c->cur_h;
     }
@@ -1355,20 +1401,16 @@ lbm_status lbm_step_record_pre(lbm_ctx* c, int n, void* f_rec, void* h_rec) {
         return fail(c, LBM_ERR_INVALID, "pre-collision records need FP32 or FP64 storage");
     DeviceGuard g(c->device);
     const size_t rsize = c->ssize;
+    lbm_status st = n > 0 ? fill_mirror_once(c) : LBM_OK;
+    if (st != LBM_OK) return st;
     for (int i = 0; i < n; ++i) {
         Buffers b = buffers(c);
         c->dp.step += 1;
         const DevParams p = c->dp;
         b.frec = (char*)f_rec + (size_t)i * flow_frec_elems(c) * rsize;
         b.hrec = (char*)h_rec + (size_t)i * c->qh * c->N * rsize;
-        cudaError_t e = fill_mirror(c, b, p);
-        if (e != cudaSuccess) return cuda_fail(c, e, "symmetry rows launch");
-        e = dispatch(c, [&](auto tag) {
-            using Tg = decltype(tag);
-            return lbmd::launch_step<typename Tg::S, Tg::Q>(b, p, c->stream, true);
-        });
+        const cudaError_t e = launch_level(c, b, p, true);
         if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
-        if ((e = zou_he_inlet(c, b, p, true)) != cudaSuccess) return cuda_fail(c, e, "inlet launch");
         c->cur_f = 1 - c->cur_f;
         c->cur_h = 1 - c->cur_h;
     }

@@ -323,8 +323,8 @@ struct DevParams {
     uint32_t mx, my;
     int sx, sy;
     uint32_t step;       // time level being written (seeds the stochastic rounding)
-    // in replayed CUDA graphs the time level is read from this device counter,
-    // which the graph advances before each step (nullptr: use step)
+    // in replayed CUDA graphs the time level is this device counter, which the
+    // graph advances at its end, plus step (nullptr: step itself)
     const uint32_t* step_ctr;
     double omega1, omega_bulk;  // f: shear and bulk rates
     double sh[7];               // h: rate of central moments of each order 0..6

@@ -58,18 +58,23 @@ constexpr int kRedBlocks = 1216;  // 8 x 152 SMs, partial sums of the reductions
 constexpr int kRedThreads = 256;
 
 // advance_h = false advances f only (velocity recomputation for the adjoint);
-// b.urec non-null records the velocity u used by each node's collision
+// b.urec non-null records the velocity u used by each node's collision.
+// walls: stream of the wall nodes' launch where the step has one (launch_plain_step),
+// forked from s and joined to it by the caller; s itself otherwise
 template <typename S, int QH>
-cudaError_t launch_step(const Buffers& b, const DevParams& p, cudaStream_t s, bool advance_h = true);
+cudaError_t launch_step(const Buffers& b, const DevParams& p, cudaStream_t s, bool advance_h, cudaStream_t walls);
 // adjoint of one level of the h evolution (R = float, or double for FP64
 // storage); h_level: the level's post-collision h record (Cumulants-1st only)
 template <typename R, int QH>
 cudaError_t launch_adjoint(const Buffers& b, const DevParams& p, const R* u_level, const R* h_level,
                            const R* mu_next, R* mu_out, AdjObjective obj, double* dtheta, cudaStream_t s);
-// Zou-He inlet plane, after a step (advance_h = false: f only)
+// Zou-He inlet plane of a step (advance_h = false: f only); it and launch_step
+// write different nodes and may run at the same time
 template <typename S, int QH>
 cudaError_t launch_inlet(const Buffers& b, const DevParams& p, cudaStream_t s, bool advance_h);
-// symmetry rows: fill them in the post-collision arrays before a step
+// whether a step leaves the symmetry rows of the level that it writes filled
+constexpr bool step_fills_symmetry(size_t ssize, int qh) { return !(ssize == 2 && qh == 27); }
+// symmetry rows: fill them in the post-collision arrays of the current level
 template <typename S, int QH>
 cudaError_t launch_mirror(const Buffers& b, const DevParams& p, cudaStream_t s);
 // out[k] = sum of acc[i * 3 + k] over i < n (the coupled adjoint's accumulators);
@@ -263,6 +268,49 @@ template <typename R> __device__ __forceinline__ R wdiv(R a, R b) {
     else return a / b;
 }
 
+// ---- symmetry rows (top and bottom symmetry planes, Sec. 4.4) -------------
+// Specular reflection at the plane halfway between a symmetry row and its
+// neighbour row: the symmetry row holds the post-collision populations of the
+// row beside it (y = 1 / y = ny-2) with e_y reversed; the step pulls from it
+// like from any node and never updates it (it is flagged solid and has no wall
+// links).  The threads of the neighbour rows write it with their own node, so
+// that no launch has to fill it before the next step (confined cylinder
+// 1000x152: k_mirror took 26.6 us and k_inlet 10.1 us of 45 us per step; 24 us
+// now).  Reads back the node's own
+// stores, which holds the rounded 16-bit values too.
+// Three rolled groups of nine populations, so that the rest of the step keeps
+// its registers.  The 16-bit D3Q27 step, which has none to spare, stays without
+// it (0.9% slower on every grid) and has the rows filled before each step.
+static __constant__ unsigned char kFlipY[27] = {
+    FLIPY(0),  FLIPY(1),  FLIPY(2),  FLIPY(3),  FLIPY(4),  FLIPY(5),  FLIPY(6),  FLIPY(7),  FLIPY(8),
+    FLIPY(9),  FLIPY(10), FLIPY(11), FLIPY(12), FLIPY(13), FLIPY(14), FLIPY(15), FLIPY(16), FLIPY(17),
+    FLIPY(18), FLIPY(19), FLIPY(20), FLIPY(21), FLIPY(22), FLIPY(23), FLIPY(24), FLIPY(25), FLIPY(26)};
+template <typename S, int Q>
+__device__ __forceinline__ void copy_flipped(S* X, int from, int to, int N) {
+    constexpr int G = Q == 27 ? 9 : 7;
+#pragma unroll 1
+    for (int i = 0; i < Q; i += G) {
+        S v[G];
+#pragma unroll
+        for (int k = 0; k < G; ++k) v[k] = X[soa(i + k, N, from)];
+#pragma unroll
+        for (int k = 0; k < G; ++k) X[soa(Q == 27 ? (int)kFlipY[i + k] : HFLIPY<7>(k), N, to)] = v[k];
+    }
+}
+template <typename S, int QH, bool DO_H>
+__device__ __forceinline__ void store_symmetry_rows(S* fB, S* hB, int n, const DevParams& p) {
+    if (!(p.mirror_lo | p.mirror_hi)) return;
+    int x, y, z;
+    node_xyz(n, p, x, y, z);
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) {
+        if (side == 0 ? !(p.mirror_lo && y == 1) : !(p.mirror_hi && y == p.ny - 2)) continue;
+        const int g = side == 0 ? n - p.nx : n + p.nx;
+        copy_flipped<S, 27>(fB, n, g, p.N);
+        if constexpr (DO_H) copy_flipped<S, QH>(hB, n, g, p.N);
+    }
+}
+
 // ---- the step: pull streaming, Eq. IBB / Eq. IABB on wall links, planes,
 // collision of f and h; one thread per node --------------------------------
 // Wall nodes find their entry in the wall table without a search: the nodes
@@ -326,6 +374,7 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH>()) k_step(const
     if (type == T_SOLID) return;
     const int N = p.N;
     if (type == T_INLET) {
+        if (p.zou_he) return;  // k_inlet writes these nodes, possibly at this moment
 #pragma unroll
         for (int a = 0; a < 27; ++a) st(fB + soa(a, N, n), inlet[a]);
         if (DO_H) {
@@ -337,6 +386,7 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH>()) k_step(const
             urec[N + n] = par<R>(p.uin[1], p.pf.uin[1]);
             urec[2 * N + n] = par<R>(p.uin[2], p.pf.uin[2]);
         }
+        if constexpr (WM != 2 && step_fills_symmetry(sizeof(S), QH)) store_symmetry_rows<S, QH, DO_H>(fB, hB, n, p);
         return;
     }
     uint32_t mask = 0;
@@ -350,7 +400,7 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH>()) k_step(const
     int x, y, z;
     node_xyz(n, p, x, y, z);
     const Nbr nb = make_nbr(x, y, z, p);
-    SrStream rs{sr_bits((uint32_t)n, p.step_ctr ? *p.step_ctr : p.step)};  // 16-bit stochastic rounding: f stores, then h
+    SrStream rs{sr_bits((uint32_t)n, (p.step_ctr ? *p.step_ctr : 0u) + p.step)};  // 16-bit stochastic rounding: f stores, then h
     R fd[27];
 #pragma unroll
     for (int a = 0; a < 27; ++a) fd[a] = ld<R>(fA + soa(a, N, src_of(nb, a)));
@@ -465,6 +515,7 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH>()) k_step(const
     }
     collide_store_h<S, QH, CUM, TRT>(hd, hB, n, p, ux, uy, uz, Q, rs);
     }
+    if constexpr (WM != 2 && step_fills_symmetry(sizeof(S), QH)) store_symmetry_rows<S, QH, DO_H>(fB, hB, n, p);
 }
 
 // With many wall nodes the plain 16-bit step runs as two launches: every
@@ -476,12 +527,15 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH>()) k_step(const
 // their pulls no longer coalesce.  Measured on the 512x256x256 porous bed
 // (D3Q7 h): FP16 22.3k -> 23.6k MLUPS; FP32 20.2k -> 20.1k, so FP32 and FP64
 // keep one launch.  Results are those of the single launch bit for bit.
+// The two write different nodes and read only the old state, so in replayed
+// graphs they run at the same time (251x127x129 bed, BF16, 42k wall nodes: the
+// wall launch alone takes 25.6 us beside 149.6 us).
 // Threshold: a wall node per LBM_WALL_SPLIT_NODES nodes or more.
 #ifndef LBM_WALL_SPLIT_NODES
 #define LBM_WALL_SPLIT_NODES 400
 #endif
 template <typename S, int QH, bool CUM, bool EQ, bool TRT>
-void launch_plain_step(const Buffers& b, const DevParams& p, cudaStream_t s) {
+void launch_plain_step(const Buffers& b, const DevParams& p, cudaStream_t s, cudaStream_t walls) {
     using R = typename Acc<S>::R;
     const int grid = (p.N + kBlock - 1) / kBlock;
 #define LBM_PLAIN_ARGS                                                                                           \
@@ -491,7 +545,7 @@ void launch_plain_step(const Buffers& b, const DevParams& p, cudaStream_t s) {
         if (p.nwall > 0 && (int64_t)p.nwall * LBM_WALL_SPLIT_NODES >= (int64_t)p.N) {
             k_step<S, QH, true, false, CUM, EQ, false, TRT, 1><<<grid, kBlock, 0, s>>>(LBM_PLAIN_ARGS);
             k_step<S, QH, true, false, CUM, EQ, false, TRT, 2>
-                <<<(p.nwall + kBlock - 1) / kBlock, kBlock, 0, s>>>(LBM_PLAIN_ARGS);
+                <<<(p.nwall + kBlock - 1) / kBlock, kBlock, 0, walls>>>(LBM_PLAIN_ARGS);
             return;
         }
     }
@@ -500,7 +554,7 @@ void launch_plain_step(const Buffers& b, const DevParams& p, cudaStream_t s) {
 }
 
 template <typename S, int QH>
-cudaError_t launch_step(const Buffers& b, const DevParams& p, cudaStream_t s, bool advance_h) {
+cudaError_t launch_step(const Buffers& b, const DevParams& p, cudaStream_t s, bool advance_h, cudaStream_t walls) {
     using R = typename Acc<S>::R;
     const int grid = (p.N + kBlock - 1) / kBlock;
     R* urec = (R*)b.urec;
@@ -532,12 +586,12 @@ cudaError_t launch_step(const Buffers& b, const DevParams& p, cudaStream_t s, bo
         const int v = (urec ? 4 : 0) | (cum ? 2 : 0) | (eq ? 1 : 0);
         switch (v) {
             case 0:
-                if (p.hkind == 0) launch_plain_step<S, QH, false, false, true>(b, p, s);
-                else launch_plain_step<S, QH, false, false, false>(b, p, s);
+                if (p.hkind == 0) launch_plain_step<S, QH, false, false, true>(b, p, s, walls);
+                else launch_plain_step<S, QH, false, false, false>(b, p, s, walls);
                 break;
-            case 1: launch_plain_step<S, QH, false, true, false>(b, p, s); break;
-            case 2: launch_plain_step<S, QH, true, false, false>(b, p, s); break;
-            case 3: launch_plain_step<S, QH, true, true, false>(b, p, s); break;
+            case 1: launch_plain_step<S, QH, false, true, false>(b, p, s, walls); break;
+            case 2: launch_plain_step<S, QH, true, false, false>(b, p, s, walls); break;
+            case 3: launch_plain_step<S, QH, true, true, false>(b, p, s, walls); break;
             case 4: k_step<S, QH, true, true, false, false><<<grid, kBlock, 0, s>>>(LBM_STEP_ARGS); break;
             case 5: k_step<S, QH, true, true, false, true><<<grid, kBlock, 0, s>>>(LBM_STEP_ARGS); break;
             case 6: k_step<S, QH, true, true, true, false><<<grid, kBlock, 0, s>>>(LBM_STEP_ARGS); break;
@@ -583,7 +637,7 @@ __global__ void __launch_bounds__(kBlock) k_init(S* __restrict__ fB, S* __restri
     R hd[QH];
     heq_dev<R, QH>(hd, (R)(rho[n] * T[n] - p.Tref) - R(0.5) * Q, vx, vy, vz, p);
     R ux, uy, uz;
-    SrStream rs{sr_bits((uint32_t)n, p.step_ctr ? *p.step_ctr : p.step)};
+    SrStream rs{sr_bits((uint32_t)n, (p.step_ctr ? *p.step_ctr : 0u) + p.step)};
     collide_store_f<S, QH>(fd, fB, n, p, ux, uy, uz, rs);
     collide_store_h<S, QH, CUM>(hd, hB, n, p, ux, uy, uz, Q, rs);
 }
@@ -1386,8 +1440,8 @@ cudaError_t launch_adjoint(const Buffers& b, const DevParams& p, const R* u_leve
 }
 
 // ---- Zou-He inlet (Sec. 4.4) ------------------------------------------------
-// Runs after the step over the inlet plane x = 0 and replaces what the step
-// stored there.  Arrivals with e_x <= 0 are pulled from the post-collision
+// Runs beside or after the step, which leaves the inlet plane x = 0 to it.
+// Arrivals with e_x <= 0 are pulled from the post-collision
 // state A as in the step.  The unknown f (e_x = +1) follow from
 // non-equilibrium bounce-back at u_in: f_a = f_abar + f^eq_a - f^eq_abar with
 // rho from mass and x-momentum, rho (1 - u_x) = sum_{e_x=0} f + 2 sum_{e_x=-1} f,
@@ -1481,7 +1535,7 @@ __global__ void __launch_bounds__(kBlock) k_inlet(const S* __restrict__ fA, S* _
         for (int a = 0; a < 27; ++a) inl[(size_t)a * p.ny * p.nz + i] = fd[a];
     }
     R vx, vy, vz;
-    SrStream rs{sr_bits((uint32_t)n, p.step_ctr ? *p.step_ctr : p.step)};
+    SrStream rs{sr_bits((uint32_t)n, (p.step_ctr ? *p.step_ctr : 0u) + p.step)};
     collide_store_f<S, QH>(fd, fB, n, p, vx, vy, vz, rs);
     if (urec) {
         urec[n] = vx;
@@ -1503,6 +1557,7 @@ __global__ void __launch_bounds__(kBlock) k_inlet(const S* __restrict__ fA, S* _
         const R Q = theta ? (R)__ldg(theta + n) : R(0);
         collide_store_h<S, QH, CUM>(hd, hB, n, p, vx, vy, vz, Q, rs);
     }
+    if constexpr (step_fills_symmetry(sizeof(S), QH)) store_symmetry_rows<S, QH, DO_H>(fB, hB, n, p);
 }
 
 template <typename S, int QH>
@@ -1519,12 +1574,9 @@ cudaError_t launch_inlet(const Buffers& b, const DevParams& p, cudaStream_t s, b
     return cudaGetLastError();
 }
 
-// ---- symmetry rows (top and bottom symmetry planes, Sec. 4.4) -------------
-// Specular reflection at the plane halfway between a symmetry row and its
-// neighbour row: before each step every node of the rows y = 0 / y = ny-1
-// takes the post-collision populations of the node beside it (y = 1 /
-// y = ny-2) with e_y reversed; the step pulls from it like from any node and
-// never writes it (it is flagged solid and has no wall links).
+// The symmetry rows of the current level, filled before the first step of a
+// call (after that each step keeps them, store_symmetry_rows): 27 + Q_h values
+// per thread, all loaded before any is stored
 template <typename S, int QH>
 __global__ void k_mirror(S* __restrict__ fA, S* __restrict__ hA, const DevParams p) {
     const int per = p.nx * p.nz;
@@ -1537,10 +1589,15 @@ __global__ void k_mirror(S* __restrict__ fA, S* __restrict__ hA, const DevParams
     const size_t N = (size_t)p.N;
     const size_t g = x + (size_t)p.nx * (yg + (size_t)p.ny * z);
     const size_t src = x + (size_t)p.nx * (ys + (size_t)p.ny * z);
+    S v[27], w[QH];
 #pragma unroll
-    for (int a = 0; a < 27; ++a) fA[a * N + g] = fA[FLIPY(a) * N + src];
+    for (int a = 0; a < 27; ++a) v[a] = fA[FLIPY(a) * N + src];
 #pragma unroll
-    for (int k = 0; k < QH; ++k) hA[k * N + g] = hA[HFLIPY<QH>(k) * N + src];
+    for (int k = 0; k < QH; ++k) w[k] = hA[HFLIPY<QH>(k) * N + src];
+#pragma unroll
+    for (int a = 0; a < 27; ++a) fA[a * N + g] = v[a];
+#pragma unroll
+    for (int k = 0; k < QH; ++k) hA[k * N + g] = w[k];
 }
 
 template <typename S, int QH>

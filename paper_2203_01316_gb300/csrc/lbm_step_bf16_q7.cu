@@ -3,7 +3,7 @@
 #include "lbm_kernels.cuh"
 
 namespace lbmd {
-template cudaError_t launch_step<__nv_bfloat16, 7>(const Buffers&, const DevParams&, cudaStream_t, bool);
+template cudaError_t launch_step<__nv_bfloat16, 7>(const Buffers&, const DevParams&, cudaStream_t, bool, cudaStream_t);
 template cudaError_t launch_objective<__nv_bfloat16, 7>(const Buffers&, const DevParams&, AdjObjective, double*, double*,
                                               cudaStream_t);
 template cudaError_t launch_init<__nv_bfloat16, 7>(const Buffers&, const DevParams&, const double*, const double*,

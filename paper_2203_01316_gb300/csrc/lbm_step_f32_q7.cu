@@ -3,7 +3,7 @@
 #include "lbm_kernels.cuh"
 
 namespace lbmd {
-template cudaError_t launch_step<float, 7>(const Buffers&, const DevParams&, cudaStream_t, bool);
+template cudaError_t launch_step<float, 7>(const Buffers&, const DevParams&, cudaStream_t, bool, cudaStream_t);
 template cudaError_t launch_objective<float, 7>(const Buffers&, const DevParams&, AdjObjective, double*, double*,
                                               cudaStream_t);
 template cudaError_t launch_init<float, 7>(const Buffers&, const DevParams&, const double*, const double*,
