@@ -333,11 +333,14 @@ __device__ __forceinline__ void store_symmetry_rows(S* fB, S* hB, int n, const D
 #ifndef LBM_STEP_MIN_BLOCKS_16
 #define LBM_STEP_MIN_BLOCKS_16 7
 #endif
-// FP64 arithmetic needs twice the registers: 2 blocks per SM
-template <typename S, int QH> constexpr int step_min_blocks() {
-    return sizeof(typename Acc<S>::R) == 8
-               ? 2
-               : (QH == 7 ? LBM_STEP_MIN_BLOCKS_Q7 : (sizeof(S) == 2 ? LBM_STEP_MIN_BLOCKS_16 : LBM_STEP_MIN_BLOCKS));
+// FP64 arithmetic needs twice the registers: 2 blocks per SM.  A step of f
+// alone holds one distribution like D3Q7 h's and takes its 8 blocks (384x128x128
+// FP32: 270 us at 96 registers -> 219 us)
+template <typename S, int QH, bool DO_H> constexpr int step_min_blocks() {
+    return sizeof(typename Acc<S>::R) == 8 ? 2
+           : (QH == 7 || !DO_H)            ? LBM_STEP_MIN_BLOCKS_Q7
+           : (sizeof(S) == 2)              ? LBM_STEP_MIN_BLOCKS_16
+                                           : LBM_STEP_MIN_BLOCKS;
 }
 
 // EQ: the BB + EQ wall rule (compile time, so the default rules keep their
@@ -347,7 +350,7 @@ template <typename S, int QH> constexpr int step_min_blocks() {
 // of the wall table (modes 1 and 2 together make one step; see launch_step)
 template <typename S, int QH, bool DO_H, bool REC, bool CUM = false, bool EQ = false, bool PRE = false,
           bool TRT = false, int WM = 0>
-__global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH>()) k_step(const S* __restrict__ fA, S* __restrict__ fB,
+__global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step(const S* __restrict__ fA, S* __restrict__ fB,
                                                   const S* __restrict__ hA, S* __restrict__ hB,
                                                   const uint8_t* __restrict__ flags,
                                                   const float* __restrict__ theta,
