@@ -205,9 +205,11 @@ class FlowObjective(torch.autograd.Function):
         s.adjoint_flow_step(None, None, muf[cur], muh[cur], muf[1 - cur], muh[1 - cur], obj0, None)
         dTw = s.adjoint_wall_gradient(ctx.n_walls, reset=True)
         dF, duin = s.adjoint_flow_gradient(reset=True)  # synchronises the solver's stream
-        gJ = gJ.detach().to(torch.float64).cpu()
-        grads = [dtheta.cpu(), torch.from_numpy(dTw), torch.from_numpy(dF), torch.from_numpy(duin)]
-        out = [(gJ * g).to(dtype=dt, device=dv) for g, (dt, dv) in zip(grads, ctx.meta)]
+        gJ = gJ.detach().to(torch.float64)
+        host = gJ.cpu()
+        # dJ/dtheta is the one of the size of the grid: it stays on the device
+        grads = [gJ.to(dev) * dtheta] + [host * torch.from_numpy(g) for g in (dTw, dF, duin)]
+        out = [g.to(dtype=dt, device=dv) for g, (dt, dv) in zip(grads, ctx.meta)]
         return out[0], out[1], out[2], out[3], None, None, None, None, None, None, None
 
 

@@ -52,7 +52,7 @@ struct lbm_ctx {
     std::vector<float> Twall{0.0f};
     float* d_theta = nullptr;
     void* d_inlet = nullptr;  // R[27 + qh]
-    double* d_scratch = nullptr;  // 3 * kRedBlocks partials + 4 results + the counter of the reductions
+    double* d_scratch = nullptr;  // kScratchDoubles
     double* d_stage = nullptr;    // 5 * N doubles for host-side outputs
     int64_t n_fluid_like = 0;     // non-solid node count
     bool geometry = false, initialised = false;
@@ -90,6 +90,10 @@ static constexpr uint8_t kMirror = 4;
 void lbm_internal_set_global_error(const std::string& msg) { g_create_err = msg; }
 
 namespace {
+
+// d_scratch: 3 * kRedBlocks partial sums, four results, the counter of the
+// reductions, the per-wall sums
+constexpr size_t kScratchDoubles = 3 * lbmd::kRedBlocks + 5 + lbmd::kWallSumMax;
 
 // every device allocation of a context goes through here (fault injection)
 template <typename T> cudaError_t dev_alloc(lbm_ctx* c, T** p, size_t bytes) {
@@ -356,14 +360,14 @@ lbm_status lbm_create(const lbm_params* params, lbm_ctx** out) {
     }
     if (dev_alloc(c, &c->d_flags, N) != cudaSuccess ||
         dev_alloc(c, &c->d_inlet, (27 + 27) * sizeof(double)) != cudaSuccess ||
-        dev_alloc(c, &c->d_scratch, (3 * lbmd::kRedBlocks + 5) * sizeof(double)) != cudaSuccess ||
+        dev_alloc(c, &c->d_scratch, kScratchDoubles * sizeof(double)) != cudaSuccess ||
         dev_alloc(c, &c->d_Twall, sizeof(float)) != cudaSuccess)
         return bail(fail(c, LBM_ERR_NOMEM, "context buffers: out of device memory"));
     if (c->ssize == 2 && dev_alloc(c, &c->d_stepctr, sizeof(uint32_t)) != cudaSuccess)
         return bail(fail(c, LBM_ERR_NOMEM, "step counter: out of device memory"));
 
     cudaMemsetAsync(c->d_flags, 0, N, c->stream);
-    cudaMemsetAsync(c->d_scratch, 0, (3 * lbmd::kRedBlocks + 5) * sizeof(double), c->stream);
+    cudaMemsetAsync(c->d_scratch, 0, kScratchDoubles * sizeof(double), c->stream);
     cudaMemsetAsync(c->d_Twall, 0, sizeof(float), c->stream);
 
     DevParams& d = c->dp;
@@ -1513,6 +1517,17 @@ lbm_status lbm_adjoint_wall_gradient(lbm_ctx* c, double* dJ_dTwall, int reset) {
     DeviceGuard g(c->device);
     for (int w = 0; w < c->n_walls; ++w) dJ_dTwall[w] = 0.0;
     if (c->nl == 0) return LBM_OK;
+    if (c->n_walls <= lbmd::kWallSumMax) {
+        double* out = c->d_scratch + 3 * lbmd::kRedBlocks + 5;
+        CK(lbmd::launch_wall_sums(c->d_dlink, c->d_lwall, c->nl, c->n_walls, c->d_scratch, out, c->stream),
+           "wall gradient launch");
+        CK(cudaMemcpyAsync(dJ_dTwall, out, c->n_walls * sizeof(double), cudaMemcpyDeviceToHost, c->stream),
+           "wall gradient copy");
+        if (reset) CK(cudaMemsetAsync(c->d_dlink, 0, c->nl * sizeof(double), c->stream), "link gradient reset");
+        CK(cudaStreamSynchronize(c->stream), "wall gradient");
+        return LBM_OK;
+    }
+    // many walls (each would scan every link): add the links on the host
     std::vector<double> acc((size_t)c->nl);
     CK(cudaMemcpyAsync(acc.data(), c->d_dlink, c->nl * sizeof(double), cudaMemcpyDeviceToHost, c->stream),
        "link gradient copy");

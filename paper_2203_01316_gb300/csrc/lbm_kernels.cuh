@@ -80,6 +80,11 @@ cudaError_t launch_mirror(const Buffers& b, const DevParams& p, cudaStream_t s);
 // out[k] = sum of acc[i * 3 + k] over i < n (the coupled adjoint's accumulators);
 // pairs: acc holds WideSum<float>
 cudaError_t launch_reduce3(const double* acc, int n, bool pairs, double* out, double* scratch, cudaStream_t s);
+// out[w] = sum of dlink[l] over the links with lwall[l] == w, for n_walls <=
+// kWallSumMax walls; part: scratch of 3 * kRedBlocks doubles, out after it
+constexpr int kWallSumMax = 64, kWallSumBlocks = 3 * kRedBlocks / kWallSumMax;
+cudaError_t launch_wall_sums(const double* dlink, const int32_t* lwall, int64_t nl, int n_walls, double* part,
+                             double* out, cudaStream_t s);
 // adjoint of one level of the coupled f + h evolution (records of the level's
 // pre-collision arrivals; f_level NULL at the initial level); wbuf: R[3][N]
 // scratch for the velocity derivative passed from the h to the f kernel

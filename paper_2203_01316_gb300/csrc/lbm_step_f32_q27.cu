@@ -74,4 +74,34 @@ cudaError_t launch_reduce3(const double* acc, int n, bool pairs, double* out, do
     else k_reduce3<<<grid, kRedThreads, 0, s>>>((const WideSum<double>*)acc, n, scratch, o);
     return cudaGetLastError();
 }
+
+// per-wall sums of the links' accumulators: blockIdx.y is the wall, a block
+// takes a stripe of the links (in a fixed order, so the sums are reproducible).
+// Copying the accumulators to pageable host memory and adding them there took
+// 0.3 ms per call at 147k links (every gradient calls it twice).
+__global__ void __launch_bounds__(kRedThreads) k_wall_sums(const double* __restrict__ dlink,
+                                                           const int32_t* __restrict__ lwall, int64_t nl,
+                                                           double* __restrict__ part) {
+    __shared__ double sh[32];
+    double v[1] = {0.0};
+    for (int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; l < nl; l += (int64_t)gridDim.x * blockDim.x)
+        if (lwall[l] == (int)blockIdx.y) v[0] += dlink[l];
+    block_sum<1>(v, sh);
+    if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = v[0];
+}
+__global__ void k_wall_sums_total(const double* __restrict__ part, int nb, double* __restrict__ out) {
+    __shared__ double sh[32];
+    double v[1] = {(int)threadIdx.x < nb ? part[blockIdx.x * nb + threadIdx.x] : 0.0};
+    block_sum<1>(v, sh);
+    if (threadIdx.x == 0) out[blockIdx.x] = v[0];
+}
+static_assert(kWallSumBlocks <= 64, "one thread per partial sum");
+
+cudaError_t launch_wall_sums(const double* dlink, const int32_t* lwall, int64_t nl, int n_walls, double* part,
+                             double* out, cudaStream_t s) {
+    const int nb = (int)std::min<int64_t>((nl + kRedThreads - 1) / kRedThreads, kWallSumBlocks);
+    k_wall_sums<<<dim3(nb, n_walls), kRedThreads, 0, s>>>(dlink, lwall, nl, part);
+    k_wall_sums_total<<<n_walls, 64, 0, s>>>(part, nb, out);
+    return cudaGetLastError();
+}
 }  // namespace lbmd

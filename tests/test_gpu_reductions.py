@@ -86,3 +86,37 @@ def test_wall_sums_of_one_and_of_many_sweeps(dims, wall_bc, qh):
     for w in range(2):
         assert abs(s.surface_flux(w) - o.surface_flux(w)) <= tol
         assert np.abs(s.wall_force(w) - o.wall_force(w)).max() <= tol
+
+
+@pytest.mark.parametrize("n_walls", [1, 3, 64, 65])
+def test_wall_temperature_gradient_of_few_and_many_walls(n_walls):
+    """dJ/dT_w summed over the links of each wall, on the device up to 64 walls and on the host beyond, against the
+    oracle's adjoint (1e-9 of the largest entry, the tolerance of the FP64 adjoint); a second gradient from reset
+    accumulators is the same."""
+    import torch
+    from oracle import oracle as O
+    from paper_2203_01316_gb300 import Solver
+    from paper_2203_01316_gb300.autograd import thermal_objective
+    nx, ny, nz = 19, 9, 11
+    N = nx * ny * nz
+    flags = I.channel_flags(nx, ny, nz, periodic_x=True)
+    links = I.plate_walls(flags, 0.3, 0.8)
+    links["wall"] = (np.arange(len(links["node"])) * 7 % n_walls).astype(np.int32)
+    Tw = list(I.uniform(4, n_walls, 0.0, 1.0).astype(np.float32).astype(np.float64))
+    fields = 1.0 + I.uniform(1, N, -1e-2, 1e-2), I.uniform(2, 3 * N, -0.05, 0.05), I.uniform(3, N, 0.0, 1.0)
+    s = Solver(nx, ny, nz, nu=0.02, k=1e-3, storage="f64", periodic_x=True)
+    o = O.Oracle(O.make_params(nx=nx, ny=ny, nz=nz, periodic_x=True, nu=0.02, k=1e-3))
+    s.set_geometry(flags.reshape(-1), links, n_walls=n_walls)
+    o.set_geometry(flags, links, nwalls=n_walls)
+    for w, T in enumerate(Tw):
+        s.set_bc(w, T)
+        o.set_wall_temperature(w, T)
+    s.init_fields(*fields)
+    state0 = s.save_state(torch.empty(s.state_size(), dtype=torch.uint8, device="cuda"))
+    f0, h0 = s.populations()
+    ref = o.adjoint(f0, h0, 5, (3, 5), ("surface", 0, 0.5), nwalls=n_walls)[2]
+    for _ in range(2):
+        theta = torch.zeros(N, dtype=torch.float64, device="cuda", requires_grad=True)
+        T = torch.tensor(Tw, dtype=torch.float64, requires_grad=True)
+        thermal_objective(theta, T, s, state0, 5, (3, 5), s.objective("surface", 0, 0.5), every=3).backward()
+        assert np.abs(T.grad.numpy() - ref).max() <= 1e-9 * np.abs(ref).max()
