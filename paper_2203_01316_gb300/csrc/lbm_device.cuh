@@ -22,6 +22,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <type_traits>
 
 namespace lbmd {
 
@@ -308,6 +309,73 @@ __host__ __device__ __forceinline__ constexpr double HALVES(int m, int n, int o)
     return (m == 2 ? 0.5 : 1.0) * (n == 2 ? 0.5 : 1.0) * (o == 2 ? 0.5 : 1.0);
 }
 
+// ---- equilibria as products, for FP64 arithmetic ----------------------------
+// GB300 issues 1.6 FP64 operations per clock and SM, so an FP64 step is bound
+// by their number (about 830 per node update with the equilibria taken through
+// the moment cube: Cumulants-1st at 256x256x1, 20 steps 2.44 ms -> 1.59 ms).
+// The equilibrium of zeroth moment psi at velocity u is psi phi_x phi_y phi_z with phi = (c_s^2 + u^2 +- u)/2
+// and 1 - c_s^2 - u^2 per axis: 12 products for the lines and one operation per
+// population.  Its difference from the reference w ref then carries the
+// rounding of the full population (1e-17 for O(0.1) values), the last place
+// of what FP64 states hold; FP32 arithmetic, whose deviations need the relative
+// precision of the moment form, does not use it.
+template <typename R> struct EqProduct {
+    R xy[9], z[3];  // psi phi_x phi_y by (e_y + 1) * 3 + e_x + 1; phi_z by e_z + 1
+    __device__ __forceinline__ EqProduct(R psi, R ux, R uy, R uz) {
+        R x[3], y[3];
+        axis(ux, x);
+        axis(uy, y);
+        axis(uz, z);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const R px = psi * x[i];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) xy[3 * j + i] = px * y[j];
+        }
+    }
+    static __device__ __forceinline__ void axis(R u, R* t) {
+        const R uu = u * u;
+        t[1] = R(2.0 / 3.0) - uu;
+        t[2] = R(0.5) * (uu + u) + R(1.0 / 6.0);
+        t[0] = t[2] - u;
+    }
+    // acc + the equilibrium of direction a
+    __device__ __forceinline__ R add(R acc, int a) const { return acc + xy[(EY(a) + 1) * 3 + EX(a) + 1] * z[EZ(a) + 1]; }
+};
+
+// inverse_cube_h of a cube that holds only the non-equilibrium part of the f
+// collision, whose z lines start with one or two moments each (the slots not
+// named in collide_f_force's list are zero and are not read)
+template <typename R>
+__device__ __forceinline__ void inverse_cube_neq(R* c, R vx, R vy, R vz) {
+    const InvAxis<R> kx = inv_axis(vx), ky = inv_axis(vy), kz = inv_axis(vz);
+#pragma unroll
+    for (int j = 0; j < 9; ++j) {
+        const int m = j % 3, n = j / 3;
+        R &lo = c[j], &mid = c[9 + j], &up = c[18 + j];
+        if ((m == 1) != (n == 1)) {  // first order in z only
+            const R k1 = mid;
+            up = kz.p1 * k1;
+            lo = kz.m1 * k1;
+            mid = -(up + lo);
+        } else if (j == 0) {  // second order in z only
+            mid = R(-2) * up;
+            lo = up;
+        } else {  // zeroth and second order
+            const R k0 = lo, k2 = up;
+            up = k2 + kz.p0 * k0;
+            lo = k2 + kz.m0 * k0;
+            mid = k0 - up - lo;
+        }
+    }
+#pragma unroll
+    for (int z = 0; z < 3; ++z)
+#pragma unroll
+        for (int x = 0; x < 3; ++x) inv3h<R>(c[9 * z + x], c[9 * z + 3 + x], c[9 * z + 6 + x], ky);
+#pragma unroll
+    for (int j = 0; j < 9; ++j) inv3h<R>(c[3 * j], c[3 * j + 1], c[3 * j + 2], kx);
+}
+
 // ---- parameters -------------------------------------------------------------
 struct DevParams {
     int nx, ny, nz, N, periodic_x;
@@ -476,8 +544,16 @@ __device__ __forceinline__ void collide_f_force(R* fd, const DevParams& p, const
                 if (m == 1 && n == 2 && o == 1) neq = n121;
                 if (m == 1 && n == 1 && o == 2) neq = n112;
                 if (m == 2 && n == 2 && o == 2) neq = n222;
-                cb[MIDX(m, n, o)] = neq + drho * Eqh<R>(m, n, o) + rho0 * Dmh<R>(m, n, o, vx, vy, vz, hx, hy, hz);
+                if constexpr (std::is_same<R, double>::value) cb[MIDX(m, n, o)] = neq;
+                else cb[MIDX(m, n, o)] = neq + drho * Eqh<R>(m, n, o) + rho0 * Dmh<R>(m, n, o, vx, vy, vz, hx, hy, hz);
             }
+    if constexpr (std::is_same<R, double>::value) {
+        inverse_cube_neq<R>(cb, vx, vy, vz);
+        const EqProduct<R> eq(rho, vx, vy, vz);
+#pragma unroll
+        for (int a = 0; a < 27; ++a) fd[a] = eq.add(cb[CUBE(a)] - rho0 * R(W27(a)), a);
+        return;
+    }
     inverse_cube_h<R>(cb, vx, vy, vz);
 #pragma unroll
     for (int a = 0; a < 27; ++a) fd[a] = cb[CUBE(a)];
@@ -593,14 +669,36 @@ __device__ __forceinline__ void heq_dev(R* hd, R dpsi, R ux, R uy, R uz, const D
 template <typename R, int QH>
 __device__ __forceinline__ void collide_h_cum(R* hd, R ux, R uy, R uz, R Q, const DevParams& p, R* m0 = nullptr) {
     R dH = 0, jx = 0, jy = 0, jz = 0;
+    if constexpr (QH == 27 && std::is_same<R, double>::value) {
+        // along x, then y, then z: 49 additions instead of 81
+        R s0[3], sx[3], sy[3];
 #pragma unroll
-    for (int i = 0; i < QH; ++i) {
-        const int a = HDIR<QH>(i);
-        const R v = hd[i];
-        dH += v;
-        if (EX(a) != 0) jx += EX(a) * v;
-        if (EY(a) != 0) jy += EY(a) * v;
-        if (EZ(a) != 0) jz += EZ(a) * v;
+        for (int k = 0; k < 3; ++k) {
+            R l0[3], l1[3];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const R a = hd[DIR(-1, j - 1, k - 1)], c = hd[DIR(1, j - 1, k - 1)];
+                l0[j] = a + c + hd[DIR(0, j - 1, k - 1)];
+                l1[j] = c - a;
+            }
+            s0[k] = l0[0] + l0[1] + l0[2];
+            sx[k] = l1[0] + l1[1] + l1[2];
+            sy[k] = l0[2] - l0[0];
+        }
+        dH = s0[0] + s0[1] + s0[2];
+        jx = sx[0] + sx[1] + sx[2];
+        jy = sy[0] + sy[1] + sy[2];
+        jz = s0[2] - s0[0];
+    } else {
+#pragma unroll
+        for (int i = 0; i < QH; ++i) {
+            const int a = HDIR<QH>(i);
+            const R v = hd[i];
+            dH += v;
+            if (EX(a) != 0) jx += EX(a) * v;
+            if (EY(a) != 0) jy += EY(a) * v;
+            if (EZ(a) != 0) jz += EZ(a) * v;
+        }
     }
     if (m0) *m0 = dH;
     const R Ht = par<R>(p.Tref, p.pf.Tref) + dH;  // zeroth moment of the stored (App. D shifted) h
@@ -651,7 +749,11 @@ __device__ __forceinline__ void feq_dev(R* fd, R drho, R ux, R uy, R uz, const D
 template <typename R, int QH>
 __device__ __forceinline__ void heq_dev(R* hd, R dpsi, R ux, R uy, R uz, const DevParams& p) {
     const R Tref = par<R>(p.Tref, p.pf.Tref);
-    if constexpr (QH == 27) {
+    if constexpr (QH == 27 && std::is_same<R, double>::value) {
+        const EqProduct<R> eq(Tref + dpsi, ux, uy, uz);
+#pragma unroll
+        for (int a = 0; a < 27; ++a) hd[a] = eq.add(-Tref * R(W27(a)), a);
+    } else if constexpr (QH == 27) {
         const R tx = ux * ux, ty = uy * uy, tz = uz * uz;
         R cb[27];
 #pragma unroll
