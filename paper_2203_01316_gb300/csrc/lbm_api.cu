@@ -295,6 +295,29 @@ template <typename T> lbm_status to_host(lbm_ctx* c, const T* src, size_t count,
 
 }  // namespace
 
+struct StateHeader {
+    char magic[8];
+    uint32_t version;
+    int32_t nx, ny, nz, qh, storage;
+    uint64_t fbytes, hbytes;
+    uint64_t step;  // time level (random stream of the 16-bit stochastic rounding)
+};
+// header and populations of a small state into device memory in one launch, by
+// elements of the storage's size (the h part starts on no wider boundary).
+// Three copies, the header's from pageable host memory, cost more than they
+// move there; the copy engines' path is as fast from a few tens of MB on:
+// box 32^3, ten steps and a copy: 102 -> 91 us
+constexpr size_t kSmallState = size_t(32) << 20;
+template <typename T>
+__global__ void k_save_small(const StateHeader hd, char* __restrict__ out, const T* __restrict__ f,
+                             const T* __restrict__ h, uint32_t nf, uint32_t nh) {
+    T* dst = (T*)(out + sizeof(StateHeader));
+    const uint32_t i0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+    for (uint32_t i = i0; i < nf + nh; i += step) dst[i] = i < nf ? f[i] : h[i - nf];
+    if (i0 < sizeof(StateHeader) / 8) ((uint64_t*)out)[i0] = ((const uint64_t*)&hd)[i0];
+}
+static_assert(sizeof(StateHeader) % 8 == 0, "copied by 8 bytes");
+
 extern "C" {
 
 lbm_status lbm_create(const lbm_params* params, lbm_ctx** out) {
@@ -1168,13 +1191,6 @@ lbm_status lbm_nusselt(lbm_ctx* c, int wall_id, double length, double area, doub
     return LBM_OK;
 }
 
-struct StateHeader {
-    char magic[8];
-    uint32_t version;
-    int32_t nx, ny, nz, qh, storage;
-    uint64_t fbytes, hbytes;
-    uint64_t step;  // time level (random stream of the 16-bit stochastic rounding)
-};
 
 lbm_status lbm_state_size(lbm_ctx* c, size_t* bytes) {
     if (!c || !bytes) return LBM_ERR_INVALID;
@@ -1204,6 +1220,21 @@ lbm_status lbm_save_state(lbm_ctx* c, void* host_buf, size_t* bytes, int is_devi
     hd.hbytes = (uint64_t)c->qh * c->N * c->ssize;
     char* out = (char*)host_buf;
     const cudaMemcpyKind kind = is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+    if (is_device && need <= kSmallState && ((uintptr_t)out & 7) == 0) {
+        const uint32_t nf = (uint32_t)27 * c->N, nh = (uint32_t)c->qh * c->N;
+        const unsigned grid = std::min<uint32_t>((nf + nh + 255) / 256, 152 * 8);
+        const void *f = c->f[c->cur_f], *h = c->h[c->cur_h];
+        if (c->ssize == 8)
+            k_save_small<<<grid, 256, 0, c->stream>>>(hd, out, (const uint64_t*)f, (const uint64_t*)h, nf, nh);
+        else if (c->ssize == 4)
+            k_save_small<<<grid, 256, 0, c->stream>>>(hd, out, (const uint32_t*)f, (const uint32_t*)h, nf, nh);
+        else
+            k_save_small<<<grid, 256, 0, c->stream>>>(hd, out, (const uint16_t*)f, (const uint16_t*)h, nf, nh);
+        CK(cudaGetLastError(), "state copy");
+        CK(cudaStreamSynchronize(c->stream), "state copy");
+        *bytes = need;
+        return LBM_OK;
+    }
     if (is_device) {
         CK(cudaMemcpyAsync(out, &hd, sizeof(hd), cudaMemcpyHostToDevice, c->stream), "state copy");
     } else {
