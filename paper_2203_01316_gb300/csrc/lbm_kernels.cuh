@@ -448,6 +448,16 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
             }
         }
     }
+    // D3Q7 h in FP32: its seven arrivals load with those of f, within the same 64
+    // registers, so that a warp waits for memory once (512x256x256 bed, 5 steps and
+    // a copy: 9.61 -> 9.34 ms).  With 27 of them the collision of f has to give up
+    // its registers (384x128x128: FP32 5.03 -> 5.26 ms, FP16 4.19 -> 4.39 ms).
+    constexpr bool H_FIRST = QH == 7 && std::is_same<S, float>::value;
+    R hd[DO_H ? QH : 1];
+    if constexpr (DO_H && H_FIRST) {
+#pragma unroll
+        for (int i = 0; i < QH; ++i) hd[i] = ld<R>(hA + soa(i, N, src_of(nb, HDIR<QH>(i))));
+    }
     R ux, uy, uz;
     if constexpr (PRE) {  // the coupled adjoint needs f only through these ten moments
         R m[10];
@@ -462,9 +472,10 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
         urec[2 * N + n] = uz;
     }
     if constexpr (DO_H) {
-    R hd[QH];
+    if constexpr (!H_FIRST) {
 #pragma unroll
-    for (int i = 0; i < QH; ++i) hd[i] = ld<R>(hA + soa(i, N, src_of(nb, HDIR<QH>(i))));
+        for (int i = 0; i < QH; ++i) hd[i] = ld<R>(hA + soa(i, N, src_of(nb, HDIR<QH>(i))));
+    }
     if (WM == 2) {  // as for f: no branches in the link bodies
         const R Tref = par<R>(p.Tref, p.pf.Tref);
 #pragma unroll
