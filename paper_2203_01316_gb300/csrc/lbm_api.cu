@@ -95,6 +95,9 @@ namespace {
 // reductions, the per-wall sums
 constexpr size_t kScratchDoubles = 3 * lbmd::kRedBlocks + 5 + lbmd::kWallSumMax;
 
+// 16-bit storage with D3Q27 h: (f_i, h_i) side by side (lbmd::paired)
+bool paired(const lbm_ctx* c) { return c->ssize == 2 && c->qh == 27; }
+
 // every device allocation of a context goes through here (fault injection)
 template <typename T> cudaError_t dev_alloc(lbm_ctx* c, T** p, size_t bytes) {
     if (c->fault_alloc > 0 && ++c->n_alloc == c->fault_alloc) {
@@ -295,6 +298,54 @@ template <typename T> lbm_status to_host(lbm_ctx* c, const T* src, size_t count,
 
 }  // namespace
 
+// paired storage <-> the state format ([27][N] f, then [27][N] h); count = 27 N
+__global__ void k_unpair(const uint32_t* __restrict__ w, unsigned short* __restrict__ f, unsigned short* __restrict__ h,
+                         uint32_t count) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= count) return;
+    const uint32_t v = w[i];
+    f[i] = (unsigned short)(v & 0xffffu);
+    h[i] = (unsigned short)(v >> 16);
+}
+__global__ void k_pair(const unsigned short* __restrict__ f, const unsigned short* __restrict__ h,
+                       uint32_t* __restrict__ w, uint32_t count) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < count) w[i] = (uint32_t)f[i] | (uint32_t)h[i] << 16;
+}
+
+// The paired state of the current level to (save) or from `buf` in the state
+// format.  Host memory, and device memory at an odd address, go through the
+// array of the other level, which holds nothing that is still needed but the
+// zeros at its solid nodes (cleared again).
+static cudaError_t copy_paired(lbm_ctx* c, char* buf, bool is_device, bool save) {
+    const uint32_t count = 27u * (uint32_t)c->N;
+    const size_t half = (size_t)count * 2;
+    uint32_t* words = (uint32_t*)c->f[c->cur_f];
+    char* other = (char*)c->f[1 - c->cur_f];
+    const bool direct = is_device && ((uintptr_t)buf & 1) == 0;
+    char* flat = direct ? buf : other;
+    const unsigned grid = (count + 255) / 256;
+    cudaError_t e = cudaSuccess;
+    if (save) {
+        k_unpair<<<grid, 256, 0, c->stream>>>(words, (unsigned short*)flat, (unsigned short*)(flat + half), count);
+        e = cudaGetLastError();
+        if (!direct && e == cudaSuccess)
+            e = cudaMemcpyAsync(buf, flat, 2 * half, is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                                c->stream);
+    } else {
+        if (!direct)
+            e = cudaMemcpyAsync(flat, buf, 2 * half, is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
+                                c->stream);
+        if (e == cudaSuccess) {
+            k_pair<<<grid, 256, 0, c->stream>>>((const unsigned short*)flat, (const unsigned short*)(flat + half), words,
+                                                count);
+            e = cudaGetLastError();
+        }
+    }
+    if (!direct && e == cudaSuccess) e = cudaMemsetAsync(other, 0, 2 * half, c->stream);
+    return e;
+}
+
 struct StateHeader {
     char magic[8];
     uint32_t version;
@@ -372,14 +423,16 @@ lbm_status lbm_create(const lbm_params* params, lbm_ctx** out) {
         if (e != cudaSuccess) return bail(cuda_fail(c, e, "stream create"));
         c->own_stream = true;
     }
-    const size_t fb = (size_t)27 * N * c->ssize, hb = (size_t)c->qh * N * c->ssize;
+    const size_t hb = paired(c) ? 0 : (size_t)c->qh * N * c->ssize;
+    const size_t fb = (size_t)(paired(c) ? 54 : 27) * N * c->ssize;
     for (int i = 0; i < 2; ++i) {
-        if (dev_alloc(c, &c->f_alloc[i], fb) != cudaSuccess || dev_alloc(c, &c->h_alloc[i], hb) != cudaSuccess)
+        if (dev_alloc(c, &c->f_alloc[i], fb) != cudaSuccess ||
+            (hb && dev_alloc(c, &c->h_alloc[i], hb) != cudaSuccess))
             return bail(fail(c, LBM_ERR_NOMEM, "population arrays: out of device memory"));
         cudaMemsetAsync(c->f_alloc[i], 0, fb, c->stream);
-        cudaMemsetAsync(c->h_alloc[i], 0, hb, c->stream);
+        if (hb) cudaMemsetAsync(c->h_alloc[i], 0, hb, c->stream);
         c->f[i] = c->f_alloc[i];
-        c->h[i] = c->h_alloc[i];
+        c->h[i] = paired(c) ? (char*)c->f_alloc[i] + c->ssize : c->h_alloc[i];
     }
     if (dev_alloc(c, &c->d_flags, N) != cudaSuccess ||
         dev_alloc(c, &c->d_inlet, (27 + 27) * sizeof(double)) != cudaSuccess ||
@@ -1220,7 +1273,7 @@ lbm_status lbm_save_state(lbm_ctx* c, void* host_buf, size_t* bytes, int is_devi
     hd.hbytes = (uint64_t)c->qh * c->N * c->ssize;
     char* out = (char*)host_buf;
     const cudaMemcpyKind kind = is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    if (is_device && need <= kSmallState && ((uintptr_t)out & 7) == 0) {
+    if (is_device && !paired(c) && need <= kSmallState && ((uintptr_t)out & 7) == 0) {
         const uint32_t nf = (uint32_t)27 * c->N, nh = (uint32_t)c->qh * c->N;
         const unsigned grid = std::min<uint32_t>((nf + nh + 255) / 256, 152 * 8);
         const void *f = c->f[c->cur_f], *h = c->h[c->cur_h];
@@ -1240,8 +1293,12 @@ lbm_status lbm_save_state(lbm_ctx* c, void* host_buf, size_t* bytes, int is_devi
     } else {
         std::memcpy(out, &hd, sizeof(hd));
     }
-    CK(cudaMemcpyAsync(out + sizeof(hd), c->f[c->cur_f], hd.fbytes, kind, c->stream), "state copy");
-    CK(cudaMemcpyAsync(out + sizeof(hd) + hd.fbytes, c->h[c->cur_h], hd.hbytes, kind, c->stream), "state copy");
+    if (paired(c)) {
+        CK(copy_paired(c, out + sizeof(hd), is_device != 0, true), "state copy");
+    } else {
+        CK(cudaMemcpyAsync(out + sizeof(hd), c->f[c->cur_f], hd.fbytes, kind, c->stream), "state copy");
+        CK(cudaMemcpyAsync(out + sizeof(hd) + hd.fbytes, c->h[c->cur_h], hd.hbytes, kind, c->stream), "state copy");
+    }
     CK(cudaStreamSynchronize(c->stream), "state copy");
     *bytes = need;
     return LBM_OK;
@@ -1265,8 +1322,12 @@ lbm_status lbm_load_state(lbm_ctx* c, const void* host_buf, size_t bytes, int is
         return fail(c, LBM_ERR_INVALID, "state does not match this context");
     const char* in = (const char*)host_buf;
     const cudaMemcpyKind kind = is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    CK(cudaMemcpyAsync(c->f[c->cur_f], in + sizeof(hd), hd.fbytes, kind, c->stream), "state load");
-    CK(cudaMemcpyAsync(c->h[c->cur_h], in + sizeof(hd) + hd.fbytes, hd.hbytes, kind, c->stream), "state load");
+    if (paired(c)) {
+        CK(copy_paired(c, const_cast<char*>(in) + sizeof(hd), is_device != 0, false), "state load");
+    } else {
+        CK(cudaMemcpyAsync(c->f[c->cur_f], in + sizeof(hd), hd.fbytes, kind, c->stream), "state load");
+        CK(cudaMemcpyAsync(c->h[c->cur_h], in + sizeof(hd) + hd.fbytes, hd.hbytes, kind, c->stream), "state load");
+    }
     CK(cudaStreamSynchronize(c->stream), "state load");
     c->dp.step = (uint32_t)hd.step;
     c->initialised = true;
@@ -1349,7 +1410,7 @@ lbm_status lbm_step_record(lbm_ctx* c, int n, void* u_rec, int advance_h) {
         const cudaError_t e = launch_level(c, b, p, advance_h != 0);
         if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
         c->cur_f = 1 - c->cur_f;
-        if (advance_h) c->cur_h = 1 - c->cur_h;
+        if (advance_h || paired(c)) c->cur_h = 1 - c->cur_h;  // (paired: h moves along with f)
     }
     return LBM_OK;
 }

@@ -80,6 +80,14 @@ template <typename R> __device__ __forceinline__ R ld(const double* p) { return 
 template <typename R> __device__ __forceinline__ R ld(const __half* p) { return (R)__half2float(__ldg(p)); }
 template <typename R> __device__ __forceinline__ R ld(const __nv_bfloat16* p) { return (R)__bfloat162float(__ldg(p)); }
 
+// the value of 16 bits of a storage type
+template <typename R> __device__ __forceinline__ R from_bits(__half*, uint32_t b) {
+    return (R)__half2float(__ushort_as_half((unsigned short)b));
+}
+template <typename R> __device__ __forceinline__ R from_bits(__nv_bfloat16*, uint32_t b) {
+    return (R)__bfloat162float(__ushort_as_bfloat16((unsigned short)b));
+}
+
 __device__ __forceinline__ void st(float* p, float v) { *p = v; }
 __device__ __forceinline__ void st(double* p, double v) { *p = v; }
 __device__ __forceinline__ void st(__half* p, float v) { *p = __float2half_rn(v); }

@@ -186,6 +186,19 @@ __device__ __forceinline__ uint32_t soa(int i, int N, int node) {
     return (uint32_t)i * (uint32_t)N + (uint32_t)node;
 }
 
+// 16-bit storage with D3Q27 h keeps f and h of one population side by side,
+// (f_i, h_i) as one 32-bit word in an array [27][N] (the h pointer is the f
+// pointer plus one element): the step reads and writes both for the same nodes,
+// so one load and one store serve the two (lbm_save_state and lbm_load_state
+// convert, their format is [27][N] f, then [27][N] h).  Two-byte accesses moved
+// half the bytes per instruction and L1 cycle: FP16 384x128x128,
+// ten steps and a copy: 4.21 -> 3.79 ms, the same bits
+template <typename S, int QH> constexpr bool paired() { return sizeof(S) == 2 && QH == 27; }
+// address of population i of a node in the f or h array X of a state
+template <typename S, int QH, typename P> __device__ __forceinline__ P* pop(P* X, int i, int N, int node) {
+    return X + (paired<S, QH>() ? 2u : 1u) * soa(i, N, node);
+}
+
 // ---- 16-bit stores ------------------------------------------------------------
 // Two values of one node (populations a and a + 1) are converted with one
 // packed conversion and stored as two 16-bit halves.  Stochastic rounding
@@ -207,28 +220,50 @@ template <bool SR> __device__ __forceinline__ uint32_t cvt_pair(__nv_bfloat16*, 
     else asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
     return d;
 }
-// v[0..Q) of node n into X[i * N + n] (16-bit storage)
+// v[0..Q) rounded to 16 bits, two per word (populations 2k and 2k + 1 in c[k])
 template <bool SR, typename S, int Q>
-__device__ __forceinline__ void store16(S* __restrict__ X, const float* v, int n, int N, SrStream& rs) {
+__device__ __forceinline__ void round16(const float* v, uint32_t* c, SrStream& rs) {
 #pragma unroll
-    for (int i = 0; i < Q; i += 2) {
-        const float hi = (i + 1 < Q) ? v[i + 1] : 0.0f;
-        const uint32_t d = cvt_pair<SR>(X, hi, v[i], SR ? rs.next() : 0u);
-        *(unsigned short*)(X + soa(i, N, n)) = (unsigned short)(d & 0xffffu);
-        if (i + 1 < Q) *(unsigned short*)(X + soa(i + 1, N, n)) = (unsigned short)(d >> 16);
-    }
+    for (int i = 0; i < Q; i += 2)
+        c[i / 2] = cvt_pair<SR>((S*)nullptr, (i + 1 < Q) ? v[i + 1] : 0.0f, v[i], SR ? rs.next() : 0u);
+}
+template <typename S, int Q>
+__device__ __forceinline__ void round16(const float* v, uint32_t* c, SrStream& rs, const DevParams& p) {
+    if (p.stochastic) round16<true, S, Q>(v, c, rs);
+    else round16<false, S, Q>(v, c, rs);
+}
+// c (from round16) of node n into X[i * N + n]
+template <typename S, int Q>
+__device__ __forceinline__ void store16(S* __restrict__ X, const uint32_t* c, int n, int N) {
+#pragma unroll
+    for (int i = 0; i < Q; ++i)
+        *(unsigned short*)(X + soa(i, N, n)) = (unsigned short)((i & 1) ? c[i / 2] >> 16 : c[i / 2] & 0xffffu);
+}
+// the words (f_i, h_i) of node n from the rounded f and h
+template <typename S>
+__device__ __forceinline__ void store_pairs(S* __restrict__ X, const uint32_t* f, const uint32_t* h, int n, int N) {
+#pragma unroll
+    for (int i = 0; i < 27; ++i)
+        ((uint32_t*)X)[soa(i, N, n)] = __byte_perm(f[i / 2], h[i / 2], (i & 1) ? 0x7632 : 0x5410);
 }
 
+// rounded f of a node on its way to the paired store (16-bit, D3Q27 h)
+struct Rounded27 {
+    uint32_t c[14];
+};
+
+// fc: paired storage keeps the rounded values there until h is known
 template <typename S, int QH>
 __device__ __forceinline__ void collide_store_f(typename Acc<S>::R* fd, S* __restrict__ fB, int n,
                                                 const DevParams& p, typename Acc<S>::R& ux,
-                                                typename Acc<S>::R& uy, typename Acc<S>::R& uz, SrStream& rs) {
+                                                typename Acc<S>::R& uy, typename Acc<S>::R& uz, SrStream& rs,
+                                                Rounded27& fc) {
     using R = typename Acc<S>::R;
     R rho;
     collide_f<R>(fd, p, ux, uy, uz, rho);
     if constexpr (sizeof(S) == 2) {
-        if (p.stochastic) store16<true, S, 27>(fB, fd, n, p.N, rs);
-        else store16<false, S, 27>(fB, fd, n, p.N, rs);
+        round16<S, 27>(fd, fc.c, rs, p);
+        if constexpr (!paired<S, QH>()) store16<S, 27>(fB, fc.c, n, p.N);
     } else {
 #pragma unroll
         for (int a = 0; a < 27; ++a) st(fB + soa(a, p.N, n), fd[a]);
@@ -236,10 +271,10 @@ __device__ __forceinline__ void collide_store_f(typename Acc<S>::R* fd, S* __res
 }
 
 template <typename S, int QH, bool CUM = false, bool TRT = false>
-__device__ __forceinline__ void collide_store_h(typename Acc<S>::R* hd, S* __restrict__ hB, int n,
+__device__ __forceinline__ void collide_store_h(typename Acc<S>::R* hd, S* __restrict__ fB, S* __restrict__ hB, int n,
                                                 const DevParams& p, typename Acc<S>::R ux,
                                                 typename Acc<S>::R uy, typename Acc<S>::R uz,
-                                                typename Acc<S>::R Q, SrStream& rs) {
+                                                typename Acc<S>::R Q, SrStream& rs, const Rounded27& fc) {
     using R = typename Acc<S>::R;
     if constexpr (sizeof(R) == 4) {
         // FP32 arithmetic: the transforms' roundings bias the zeroth moment of
@@ -256,12 +291,24 @@ __device__ __forceinline__ void collide_store_h(typename Acc<S>::R* hd, S* __res
         collide_h<R, QH, CUM, TRT>(hd, ux, uy, uz, Q, p);
     }
     if constexpr (sizeof(S) == 2) {
-        if (p.stochastic) store16<true, S, QH>(hB, hd, n, p.N, rs);
-        else store16<false, S, QH>(hB, hd, n, p.N, rs);
+        uint32_t c[(QH + 1) / 2];
+        round16<S, QH>(hd, c, rs, p);
+        if constexpr (paired<S, QH>()) store_pairs<S>(fB, fc.c, c, n, p.N);
+        else store16<S, QH>(hB, c, n, p.N);
     } else {
 #pragma unroll
         for (int i = 0; i < QH; ++i) st(hB + soa(i, p.N, n), hd[i]);
     }
+}
+
+// paired storage, a step that advances f only: the node's h moves along
+template <typename S>
+__device__ __forceinline__ void store_f_keep_h(const S* __restrict__ fA, S* __restrict__ fB, const Rounded27& fc, int n,
+                                               int N) {
+#pragma unroll
+    for (int i = 0; i < 27; ++i)
+        ((uint32_t*)fB)[soa(i, N, n)] =
+            __byte_perm(fc.c[i / 2], __ldg((const uint32_t*)fA + soa(i, N, n)), (i & 1) ? 0x7632 : 0x7610);
 }
 
 // the division of the q > 1/2 link rule: the denominator 2q lies in [1, 2],
@@ -290,16 +337,16 @@ static __constant__ unsigned char kFlipY[27] = {
     FLIPY(0),  FLIPY(1),  FLIPY(2),  FLIPY(3),  FLIPY(4),  FLIPY(5),  FLIPY(6),  FLIPY(7),  FLIPY(8),
     FLIPY(9),  FLIPY(10), FLIPY(11), FLIPY(12), FLIPY(13), FLIPY(14), FLIPY(15), FLIPY(16), FLIPY(17),
     FLIPY(18), FLIPY(19), FLIPY(20), FLIPY(21), FLIPY(22), FLIPY(23), FLIPY(24), FLIPY(25), FLIPY(26)};
-template <typename S, int Q>
+template <typename S, int Q, uint32_t P>  // P: elements per population of a node
 __device__ __forceinline__ void copy_flipped(S* X, int from, int to, int N) {
     constexpr int G = Q == 27 ? 9 : 7;
 #pragma unroll 1
     for (int i = 0; i < Q; i += G) {
         S v[G];
 #pragma unroll
-        for (int k = 0; k < G; ++k) v[k] = X[soa(i + k, N, from)];
+        for (int k = 0; k < G; ++k) v[k] = X[P * soa(i + k, N, from)];
 #pragma unroll
-        for (int k = 0; k < G; ++k) X[soa(Q == 27 ? (int)kFlipY[i + k] : HFLIPY<7>(k), N, to)] = v[k];
+        for (int k = 0; k < G; ++k) X[P * soa(Q == 27 ? (int)kFlipY[i + k] : HFLIPY<7>(k), N, to)] = v[k];
     }
 }
 template <typename S, int QH, bool DO_H>
@@ -311,8 +358,8 @@ __device__ __forceinline__ void store_symmetry_rows(S* fB, S* hB, int n, const D
     for (int side = 0; side < 2; ++side) {
         if (side == 0 ? !(p.mirror_lo && y == 1) : !(p.mirror_hi && y == p.ny - 2)) continue;
         const int g = side == 0 ? n - p.nx : n + p.nx;
-        copy_flipped<S, 27>(fB, n, g, p.N);
-        if constexpr (DO_H) copy_flipped<S, QH>(hB, n, g, p.N);
+        copy_flipped<S, 27, paired<S, QH>() ? 2u : 1u>(fB, n, g, p.N);
+        if constexpr (DO_H) copy_flipped<S, QH, paired<S, QH>() ? 2u : 1u>(hB, n, g, p.N);
     }
 }
 
@@ -384,17 +431,20 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
     if (type == T_INLET) {
         if (p.zou_he) return;  // k_inlet writes these nodes, possibly at this moment
 #pragma unroll
-        for (int a = 0; a < 27; ++a) st(fB + soa(a, N, n), inlet[a]);
-        if (DO_H) {
+        for (int a = 0; a < 27; ++a) st(pop<S, QH>(fB, a, N, n), inlet[a]);
+        if (DO_H || paired<S, QH>()) {
 #pragma unroll
-            for (int i = 0; i < QH; ++i) st(hB + soa(i, N, n), inlet[27 + i]);
+            for (int i = 0; i < QH; ++i) {
+                if constexpr (DO_H) st(pop<S, QH>(hB, i, N, n), inlet[27 + i]);
+                else *pop<S, QH>(hB, i, N, n) = *pop<S, QH>(hA, i, N, n);
+            }
         }
         if (REC) {
             urec[n] = par<R>(p.uin[0], p.pf.uin[0]);
             urec[N + n] = par<R>(p.uin[1], p.pf.uin[1]);
             urec[2 * N + n] = par<R>(p.uin[2], p.pf.uin[2]);
         }
-        if constexpr (WM != 2 && step_fills_symmetry(sizeof(S), QH)) store_symmetry_rows<S, QH, DO_H>(fB, hB, n, p);
+        if constexpr (WM != 2 && step_fills_symmetry(sizeof(S), QH)) store_symmetry_rows<S, QH, DO_H || paired<S, QH>()>(fB, hB, n, p);
         return;
     }
     uint32_t mask = 0;
@@ -410,8 +460,16 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
     const Nbr nb = make_nbr(x, y, z, p);
     SrStream rs{sr_bits((uint32_t)n, (p.step_ctr ? *p.step_ctr : 0u) + p.step)};  // 16-bit stochastic rounding: f stores, then h
     R fd[27];
+    uint32_t word[paired<S, QH>() ? 27 : 1];  // paired storage: (f, h) of each arrival
+    if constexpr (paired<S, QH>()) {
 #pragma unroll
-    for (int a = 0; a < 27; ++a) fd[a] = ld<R>(fA + soa(a, N, src_of(nb, a)));
+        for (int a = 0; a < 27; ++a) word[a] = __ldg((const uint32_t*)fA + soa(a, N, src_of(nb, a)));
+#pragma unroll
+        for (int a = 0; a < 27; ++a) fd[a] = from_bits<R>((S*)nullptr, word[a] & 0xffffu);
+    } else {
+#pragma unroll
+        for (int a = 0; a < 27; ++a) fd[a] = ld<R>(fA + soa(a, N, src_of(nb, a)));
+    }
     if (WM == 2) {
         // wall nodes alone, so every lane has links: the link bodies without
         // branches (loads predicated on the mask bit, the result selected),
@@ -422,8 +480,8 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
             const bool has = (mask >> a) & 1u;
             const float q = has ? __ldg(lq + off + __popc(mask & ((1u << a) - 1u))) : 0.5f;
             const bool thin = (mask >> b) & 1u;
-            const R fa_b = has ? ld<R>(fA + soa(a, N, n)) : R(0);
-            const R fb_b = has ? ld<R>(fA + soa(b, N, n)) : R(0);
+            const R fa_b = has ? ld<R>(pop<S, QH>(fA, a, N, n)) : R(0);
+            const R fb_b = has ? ld<R>(pop<S, QH>(fA, b, N, n)) : R(0);
             const R qq = (R)fmaxf(q, 0.5f);
             const R v_lin = R(2) * (R)q * fa_b + (R(1) - R(2) * (R)q) * fd[a];
             const R v_far = wdiv<R>(fa_b + (R(2) * qq - R(1)) * fb_b, R(2) * qq);
@@ -438,12 +496,12 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
             if (!(mask & (1u << a))) continue;
             const float q = __ldg(lq + off + __popc(mask & ((1u << a) - 1u)));
             const bool thin = (mask >> b) & 1u;  // x_f = x_b - e_a is solid too
-            const R fa_b = ld<R>(fA + soa(a, N, n));
+            const R fa_b = ld<R>(pop<S, QH>(fA, a, N, n));
             if (q <= 0.5f && !thin) {
                 fd[b] = R(2) * (R)q * fa_b + (R(1) - R(2) * (R)q) * fd[a];  // fd[a] = f*_a(x_f)
             } else {
                 const R qq = (R)fmaxf(q, 0.5f);
-                const R fb_b = ld<R>(fA + soa(b, N, n));
+                const R fb_b = ld<R>(pop<S, QH>(fA, b, N, n));
                 fd[b] = wdiv<R>(fa_b + (R(2) * qq - R(1)) * fb_b, R(2) * qq);
             }
         }
@@ -456,7 +514,7 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
     R hd[DO_H ? QH : 1];
     if constexpr (DO_H && H_FIRST) {
 #pragma unroll
-        for (int i = 0; i < QH; ++i) hd[i] = ld<R>(hA + soa(i, N, src_of(nb, HDIR<QH>(i))));
+        for (int i = 0; i < QH; ++i) hd[i] = ld<R>(pop<S, QH>(hA, i, N, src_of(nb, HDIR<QH>(i))));
     }
     R ux, uy, uz;
     if constexpr (PRE) {  // the coupled adjoint needs f only through these ten moments
@@ -465,14 +523,19 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
 #pragma unroll
         for (int k = 0; k < 10; ++k) ((R*)frec)[soa(k, N, n)] = m[k];
     }
-    collide_store_f<S, QH>(fd, fB, n, p, ux, uy, uz, rs);
+    Rounded27 fc;
+    collide_store_f<S, QH>(fd, fB, n, p, ux, uy, uz, rs, fc);
+    if constexpr (!DO_H && paired<S, QH>()) store_f_keep_h<S>(fA, fB, fc, n, N);
     if (REC) {
         urec[n] = ux;
         urec[N + n] = uy;
         urec[2 * N + n] = uz;
     }
     if constexpr (DO_H) {
-    if constexpr (!H_FIRST) {
+    if constexpr (paired<S, QH>()) {
+#pragma unroll
+        for (int i = 0; i < QH; ++i) hd[i] = from_bits<R>((S*)nullptr, word[i] >> 16);
+    } else if constexpr (!H_FIRST) {
 #pragma unroll
         for (int i = 0; i < QH; ++i) hd[i] = ld<R>(hA + soa(i, N, src_of(nb, HDIR<QH>(i))));
     }
@@ -492,8 +555,8 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
             if constexpr (EQ) {
                 v = R(0.5) * heq2;
             } else {
-                const R ha_b = has ? ld<R>(hA + soa(ia, N, n)) : R(0);
-                const R hb_b = has ? ld<R>(hA + soa(ib, N, n)) : R(0);
+                const R ha_b = has ? ld<R>(pop<S, QH>(hA, ia, N, n)) : R(0);
+                const R hb_b = has ? ld<R>(pop<S, QH>(hA, ib, N, n)) : R(0);
                 const R qq = (R)fmaxf(q, 0.5f);
                 const R v_lin = -(R(2) * (R)q * ha_b + (R(1) - R(2) * (R)q) * hd[ia]) + heq2;
                 const R v_far = wdiv<R>(-ha_b + (R(2) * qq - R(1)) * hb_b + heq2, R(2) * qq);
@@ -517,12 +580,12 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
                 hd[ib] = R(0.5) * heq2;
                 continue;
             }
-            const R ha_b = ld<R>(hA + soa(ia, N, n));
+            const R ha_b = ld<R>(pop<S, QH>(hA, ia, N, n));
             if (q <= 0.5f && !thin) {
                 hd[ib] = -(R(2) * (R)q * ha_b + (R(1) - R(2) * (R)q) * hd[ia]) + heq2;
             } else {
                 const R qq = (R)fmaxf(q, 0.5f);
-                const R hb_b = ld<R>(hA + soa(ib, N, n));
+                const R hb_b = ld<R>(pop<S, QH>(hA, ib, N, n));
                 hd[ib] = wdiv<R>(-ha_b + (R(2) * qq - R(1)) * hb_b + heq2, R(2) * qq);
             }
         }
@@ -532,9 +595,9 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
 #pragma unroll
         for (int i = 0; i < QH; ++i) ((R*)hrec)[soa(i, N, n)] = hd[i];
     }
-    collide_store_h<S, QH, CUM, TRT>(hd, hB, n, p, ux, uy, uz, Q, rs);
+    collide_store_h<S, QH, CUM, TRT>(hd, fB, hB, n, p, ux, uy, uz, Q, rs, fc);
     }
-    if constexpr (WM != 2 && step_fills_symmetry(sizeof(S), QH)) store_symmetry_rows<S, QH, DO_H>(fB, hB, n, p);
+    if constexpr (WM != 2 && step_fills_symmetry(sizeof(S), QH)) store_symmetry_rows<S, QH, DO_H || paired<S, QH>()>(fB, hB, n, p);
 }
 
 // With many wall nodes the plain 16-bit step runs as two launches: every
@@ -636,16 +699,16 @@ __global__ void __launch_bounds__(kBlock) k_init(S* __restrict__ fB, S* __restri
     const int type = flags[n] & 3;
     if (type == T_SOLID) {
 #pragma unroll
-        for (int a = 0; a < 27; ++a) st(fB + (size_t)a * p.N + n, R(0));
+        for (int a = 0; a < 27; ++a) st(pop<S, QH>(fB, a, p.N, n), R(0));
 #pragma unroll
-        for (int i = 0; i < QH; ++i) st(hB + (size_t)i * p.N + n, R(0));
+        for (int i = 0; i < QH; ++i) st(pop<S, QH>(hB, i, p.N, n), R(0));
         return;
     }
     if (type == T_INLET) {
 #pragma unroll
-        for (int a = 0; a < 27; ++a) st(fB + (size_t)a * p.N + n, inlet[a]);
+        for (int a = 0; a < 27; ++a) st(pop<S, QH>(fB, a, p.N, n), inlet[a]);
 #pragma unroll
-        for (int i = 0; i < QH; ++i) st(hB + (size_t)i * p.N + n, inlet[27 + i]);
+        for (int i = 0; i < QH; ++i) st(pop<S, QH>(hB, i, p.N, n), inlet[27 + i]);
         return;
     }
     const R vx = (R)u[n], vy = (R)u[(size_t)p.N + n], vz = (R)u[2 * (size_t)p.N + n];
@@ -657,8 +720,9 @@ __global__ void __launch_bounds__(kBlock) k_init(S* __restrict__ fB, S* __restri
     heq_dev<R, QH>(hd, (R)(rho[n] * T[n] - p.Tref) - R(0.5) * Q, vx, vy, vz, p);
     R ux, uy, uz;
     SrStream rs{sr_bits((uint32_t)n, (p.step_ctr ? *p.step_ctr : 0u) + p.step)};
-    collide_store_f<S, QH>(fd, fB, n, p, ux, uy, uz, rs);
-    collide_store_h<S, QH, CUM>(hd, hB, n, p, ux, uy, uz, Q, rs);
+    Rounded27 fc;
+    collide_store_f<S, QH>(fd, fB, n, p, ux, uy, uz, rs, fc);
+    collide_store_h<S, QH, CUM>(hd, fB, hB, n, p, ux, uy, uz, Q, rs, fc);
 }
 
 template <typename S, int QH>
@@ -698,14 +762,14 @@ __global__ void k_macros(const S* __restrict__ fA, const S* __restrict__ hA, con
     R dr = 0, jx = 0, jy = 0, jz = 0, dh = 0;
 #pragma unroll
     for (int a = 0; a < 27; ++a) {
-        const R v = ld<R>(fA + a * N + n);
+        const R v = ld<R>(pop<S, QH>(fA, a, p.N, n));
         dr += v;
         jx += EX(a) * v;
         jy += EY(a) * v;
         jz += EZ(a) * v;
     }
 #pragma unroll
-    for (int i = 0; i < QH; ++i) dh += ld<R>(hA + i * N + n);
+    for (int i = 0; i < QH; ++i) dh += ld<R>(pop<S, QH>(hA, i, p.N, n));
     const R r = par<R>(p.rho0, p.pf.rho0) + dr;
     const R Q = theta ? (R)theta[n] : R(0);
     rho[n] = (double)r;
@@ -733,12 +797,12 @@ __global__ void k_populations(const S* __restrict__ fA, const S* __restrict__ hA
     if (f) {
 #pragma unroll
         for (int a = 0; a < 27; ++a)
-            f[a * N + n] = solid ? 0.0 : (double)ld<R>(fA + a * N + n) + W27(a) * p.rho0;
+            f[a * N + n] = solid ? 0.0 : (double)ld<R>(pop<S, QH>(fA, a, p.N, n)) + W27(a) * p.rho0;
     }
     if (h) {
 #pragma unroll
         for (int i = 0; i < QH; ++i)
-            h[i * N + n] = solid ? 0.0 : (double)ld<R>(hA + i * N + n) + HW<QH>(i) * p.Tref;
+            h[i * N + n] = solid ? 0.0 : (double)ld<R>(pop<S, QH>(hA, i, p.N, n)) + HW<QH>(i) * p.Tref;
     }
 }
 
@@ -805,21 +869,21 @@ __global__ void __launch_bounds__(kRedThreads) k_balances(const S* __restrict__ 
         // a node's values are added as wide sums, the nodes in FP64
         WideSum<R> sumf, sumh;
 #pragma unroll
-        for (int a = 0; a < 27; ++a) sumf.add(ld<R>(fA + a * N + n));
+        for (int a = 0; a < 27; ++a) sumf.add(ld<R>(pop<S, QH>(fA, a, p.N, n)));
 #pragma unroll
-        for (int i = 0; i < QH; ++i) sumh.add(ld<R>(hA + i * N + n));
+        for (int i = 0; i < QH; ++i) sumh.add(ld<R>(pop<S, QH>(hA, i, p.N, n)));
         if (isfinite(sumf.hi) && isfinite(sumh.hi)) {
             v[0] += sumf.value();
             v[1] += sumh.value();
         } else {  // a non-finite value, or a sum beyond the float range: one by one in FP64
             bool bad = false;
             for (int a = 0; a < 27; ++a) {
-                const R x = ld<R>(fA + a * N + n);
+                const R x = ld<R>(pop<S, QH>(fA, a, p.N, n));
                 bad |= !isfinite(x);
                 v[0] += (double)x;
             }
             for (int i = 0; i < QH; ++i) {
-                const R x = ld<R>(hA + i * N + n);
+                const R x = ld<R>(pop<S, QH>(hA, i, p.N, n));
                 bad |= !isfinite(x);
                 v[1] += (double)x;
             }
@@ -975,18 +1039,18 @@ __global__ void __launch_bounds__(kRedThreads) k_surface_flux(const S* __restric
         const int n = wnode[w];
         const float q = lq[l];
         const bool thin = (mask >> d.b) & 1u;
-        const R ha_b = ld<R>(hA + ia * N + n);
+        const R ha_b = ld<R>(pop<S, QH>(hA, ia, p.N, n));
         R hin;
         if (p.wall_bc == 1) {
             hin = R(0.5) * heq2;
         } else if (q <= 0.5f && !thin) {
             int x, y, z;
             node_xyz(n, p, x, y, z);
-            const R ha_f = ld<R>(hA + ia * N + lane_src(d, x, y, z, p));
+            const R ha_f = ld<R>(pop<S, QH>(hA, ia, p.N, lane_src(d, x, y, z, p)));
             hin = -(R(2) * (R)q * ha_b + (R(1) - R(2) * (R)q) * ha_f) + heq2;
         } else {
             const R qq = (R)fmaxf(q, 0.5f);
-            const R hb_b = ld<R>(hA + ib * N + n);
+            const R hb_b = ld<R>(pop<S, QH>(hA, ib, p.N, n));
             hin = (-ha_b + (R(2) * qq - R(1)) * hb_b + heq2) / (R(2) * qq);
         }
         sum.add(hin);
@@ -1013,7 +1077,7 @@ cudaError_t launch_surface_flux(const Buffers& b, const DevParams& p, int wall, 
 // the paper): every link (x_b, a) of the wall carries e_a f*_a(x_b, t) into
 // the wall and takes back e_a f_abar(x_b, t+1) from Eq. IBB, exactly as the
 // step applies it; the stored deviations add 2 w_a rho0 per link
-template <typename S>
+template <typename S, int QH>
 __global__ void __launch_bounds__(kRedThreads) k_wall_force(const S* __restrict__ fA,
                                                             const int32_t* __restrict__ wnode,
                                                             const uint32_t* __restrict__ wmask,
@@ -1039,15 +1103,15 @@ __global__ void __launch_bounds__(kRedThreads) k_wall_force(const S* __restrict_
         const int n = wnode[w];
         const float q = lq[l];
         const bool thin = (mask >> d.b) & 1u;  // x_f = x_b - e_a is solid
-        const R fa_b = ld<R>(fA + d.a * N + n);
+        const R fa_b = ld<R>(pop<S, QH>(fA, d.a, p.N, n));
         R fin;
         if (q <= 0.5f && !thin) {
             int x, y, z;
             node_xyz(n, p, x, y, z);
-            fin = R(2) * (R)q * fa_b + (R(1) - R(2) * (R)q) * ld<R>(fA + d.a * N + lane_src(d, x, y, z, p));
+            fin = R(2) * (R)q * fa_b + (R(1) - R(2) * (R)q) * ld<R>(pop<S, QH>(fA, d.a, p.N, lane_src(d, x, y, z, p)));
         } else {
             const R qq = (R)fmaxf(q, 0.5f);
-            fin = (fa_b + (R(2) * qq - R(1)) * ld<R>(fA + d.b * N + n)) / (R(2) * qq);
+            fin = (fa_b + (R(2) * qq - R(1)) * ld<R>(pop<S, QH>(fA, d.b, p.N, n))) / (R(2) * qq);
         }
         sum.add(fa_b);
         sum.add(fin);
@@ -1058,17 +1122,17 @@ __global__ void __launch_bounds__(kRedThreads) k_wall_force(const S* __restrict_
     if (reduce_in_last_block<3>(v, sh, part, red_counter(part))) write_totals<3>(v, o);
 }
 
-template <typename S>
+template <typename S, int QH>
 cudaError_t wall_force_to(const Buffers& b, const DevParams& p, int wall, double* scratch, const RedOut& o,
                           cudaStream_t s) {
-    k_wall_force<S><<<wall_blocks(b.nw, kWallLanes27), kRedThreads, 0, s>>>(
+    k_wall_force<S, QH><<<wall_blocks(b.nw, kWallLanes27), kRedThreads, 0, s>>>(
         (const S*)b.fA, b.wnode, b.wmask, b.woff, b.lq, b.lwall, b.nw, wall, scratch, o, p);
     return cudaGetLastError();
 }
 template <typename S, int QH>
 cudaError_t launch_wall_force(const Buffers& b, const DevParams& p, int wall, double* scratch, double* out,
                               cudaStream_t s) {
-    return wall_force_to<S>(b, p, wall, scratch, RedOut{out, nullptr, 0.0, 0}, s);
+    return wall_force_to<S, QH>(b, p, wall, scratch, RedOut{out, nullptr, 0.0, 0}, s);
 }
 
 // ---- adjoint of the h evolution --------------------------------------------
@@ -1542,7 +1606,7 @@ __global__ void __launch_bounds__(kBlock) k_inlet(const S* __restrict__ fA, S* _
     const R ux = par<R>(p.uin[0], p.pf.uin[0]), uy = par<R>(p.uin[1], p.pf.uin[1]), uz = par<R>(p.uin[2], p.pf.uin[2]);
     R fd[27];
 #pragma unroll
-    for (int a = 0; a < 27; ++a) fd[a] = (EX(a) == 1) ? R(0) : ld<R>(fA + a * N + src_of(nb, a));
+    for (int a = 0; a < 27; ++a) fd[a] = (EX(a) == 1) ? R(0) : ld<R>(pop<S, QH>(fA, a, p.N, src_of(nb, a)));
     const R drho = zou_he_fill_f<R>(fd, ux, uy, uz, p);
     if (frec) {
         R m[10];
@@ -1555,7 +1619,9 @@ __global__ void __launch_bounds__(kBlock) k_inlet(const S* __restrict__ fA, S* _
     }
     R vx, vy, vz;
     SrStream rs{sr_bits((uint32_t)n, (p.step_ctr ? *p.step_ctr : 0u) + p.step)};
-    collide_store_f<S, QH>(fd, fB, n, p, vx, vy, vz, rs);
+    Rounded27 fc;
+    collide_store_f<S, QH>(fd, fB, n, p, vx, vy, vz, rs, fc);
+    if constexpr (!DO_H && paired<S, QH>()) store_f_keep_h<S>(fA, fB, fc, n, N);
     if (urec) {
         urec[n] = vx;
         urec[N + n] = vy;
@@ -1566,7 +1632,7 @@ __global__ void __launch_bounds__(kBlock) k_inlet(const S* __restrict__ fA, S* _
 #pragma unroll
         for (int k = 0; k < QH; ++k) {
             const int a = HDIR<QH>(k);
-            hd[k] = (EX(a) == 1) ? R(0) : ld<R>(hA + k * N + src_of(nb, a));
+            hd[k] = (EX(a) == 1) ? R(0) : ld<R>(pop<S, QH>(hA, k, p.N, src_of(nb, a)));
         }
         zou_he_fill_h<R, QH>(hd, drho, ux, uy, uz, p);
         if (hrec) {
@@ -1574,9 +1640,9 @@ __global__ void __launch_bounds__(kBlock) k_inlet(const S* __restrict__ fA, S* _
             for (int k = 0; k < QH; ++k) ((R*)hrec)[k * N + n] = hd[k];
         }
         const R Q = theta ? (R)__ldg(theta + n) : R(0);
-        collide_store_h<S, QH, CUM>(hd, hB, n, p, vx, vy, vz, Q, rs);
+        collide_store_h<S, QH, CUM>(hd, fB, hB, n, p, vx, vy, vz, Q, rs, fc);
     }
-    if constexpr (step_fills_symmetry(sizeof(S), QH)) store_symmetry_rows<S, QH, DO_H>(fB, hB, n, p);
+    if constexpr (step_fills_symmetry(sizeof(S), QH)) store_symmetry_rows<S, QH, DO_H || paired<S, QH>()>(fB, hB, n, p);
 }
 
 template <typename S, int QH>
@@ -1610,13 +1676,13 @@ __global__ void k_mirror(S* __restrict__ fA, S* __restrict__ hA, const DevParams
     const size_t src = x + (size_t)p.nx * (ys + (size_t)p.ny * z);
     S v[27], w[QH];
 #pragma unroll
-    for (int a = 0; a < 27; ++a) v[a] = fA[FLIPY(a) * N + src];
+    for (int a = 0; a < 27; ++a) v[a] = *pop<S, QH>(fA, FLIPY(a), p.N, (int)src);
 #pragma unroll
-    for (int k = 0; k < QH; ++k) w[k] = hA[HFLIPY<QH>(k) * N + src];
+    for (int k = 0; k < QH; ++k) w[k] = *pop<S, QH>(hA, HFLIPY<QH>(k), p.N, (int)src);
 #pragma unroll
-    for (int a = 0; a < 27; ++a) fA[a * N + g] = v[a];
+    for (int a = 0; a < 27; ++a) *pop<S, QH>(fA, a, p.N, (int)g) = v[a];
 #pragma unroll
-    for (int k = 0; k < QH; ++k) hA[k * N + g] = w[k];
+    for (int k = 0; k < QH; ++k) *pop<S, QH>(hA, k, p.N, (int)g) = w[k];
 }
 
 template <typename S, int QH>
@@ -2478,7 +2544,7 @@ __global__ void k_record_h(const S* __restrict__ hA, typename Acc<S>::R* __restr
     using R = typename Acc<S>::R;
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (size_t)QH * p.N) return;
-    rec[i] = ld<R>(hA + i);
+    rec[i] = ld<R>(hA + (paired<S, QH>() ? 2 * i : i));
 }
 
 template <typename S, int QH>
@@ -2507,7 +2573,7 @@ __global__ void __launch_bounds__(kRedThreads) k_section_flux(const S* __restric
 #pragma unroll
         for (int i = 0; i < QH; ++i) {
             const int ex = EX(HDIR<QH>(i));
-            if (ex != 0) v[0] += (double)ex * (double)ld<R>(hA + i * N + n);
+            if (ex != 0) v[0] += (double)ex * (double)ld<R>(pop<S, QH>(hA, i, p.N, n));
         }
     }
     if (reduce_in_last_block<1>(v, sh, part, red_counter(part))) write_totals<1>(v, o);
@@ -2517,7 +2583,7 @@ template <typename S, int QH>
 cudaError_t launch_objective(const Buffers& b, const DevParams& p, AdjObjective obj, double* scratch, double* acc,
                              cudaStream_t s) {
     const RedOut o{nullptr, acc, obj.weight, obj.kind == 2 ? obj.comp : 0};
-    if (obj.kind == 2) return wall_force_to<S>(b, p, obj.wall, scratch, o, s);
+    if (obj.kind == 2) return wall_force_to<S, QH>(b, p, obj.wall, scratch, o, s);
     if (obj.kind == 0) return surface_flux_to<S, QH>(b, p, obj.wall, scratch, o, s);
     const int rows = p.ny * p.nz;
     k_section_flux<S, QH><<<std::min((rows + kRedThreads - 1) / kRedThreads, kRedBlocks), kRedThreads, 0, s>>>(
