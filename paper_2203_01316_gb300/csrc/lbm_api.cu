@@ -355,9 +355,9 @@ struct StateHeader {
 };
 // header and populations of a small state into device memory in one launch, by
 // elements of the storage's size (the h part starts on no wider boundary).
-// Three copies, the header's from pageable host memory, cost more than they
-// move there; the copy engines' path is as fast from a few tens of MB on:
-// box 32^3, ten steps and a copy: 102 -> 91 us
+// Three copies, the header's from pageable host memory, cost more than what
+// they move there (box 32^3, ten steps and a copy: 102 -> 91 us); at 32 MiB the
+// bytes take about 10 us, and larger states keep the copies.
 constexpr size_t kSmallState = size_t(32) << 20;
 template <typename T>
 __global__ void k_save_small(const StateHeader hd, char* __restrict__ out, const T* __restrict__ f,

@@ -907,9 +907,10 @@ cudaError_t launch_balances(const Buffers& b, const DevParams& p, double* scratc
 // ---- wall sums: one lane per link ---------------------------------------------
 // A group of lanes takes one wall node, lane i its direction i, so that the
 // links of a node load together; a thread that walked its node's links one
-// after another waited for each link's loads in turn (384x128x128 sphere: flux
-// 34 us, force 44 us and two reductions of 5 us; fields, totals, flux and force
-// of that state 764 -> 711 us).  Each lane keeps one direction throughout, so the links' values
+// after another waited for each link's loads in turn (128x64x64 plate channel:
+// flux 34 us and a reduction of 5 us -> 11 us; 384x128x128 sphere: force 44 us
+// and 5 us -> 25 us; fields, totals, flux and force of that state 764 -> 711 us).
+// Each lane keeps one direction throughout, so the links' values
 // are added as a WideSum and multiplied by the lane's constants once at the end.
 constexpr int kWallLanes27 = 32, kWallLanes7 = 8;
 template <int QH> constexpr int wall_lanes() { return QH == 27 ? kWallLanes27 : kWallLanes7; }
@@ -2438,8 +2439,10 @@ __device__ __forceinline__ void adjoint_flow_node(
 // row.  Each slot has one owner, so there are no atomics.  One FP64 slot of six
 // per node took 96 B of the f part's 460 B per node, six operations a node on
 // the FP64 pipe, and 1.4 ms to add up at 192x64x64 (60 levels and their
-// recomputation there: 26.30 -> 22.36 ms, with dJ/dQ as WideSum, which took the
-// h part from 102 to 93 us)
+// recomputation there: 26.30 -> 22.36 ms, with dJ/dQ as WideSum).  Both parts
+// wait on their loads: h 79 us at 80 registers (24 warps per SM), f 61 us at 72
+// (28 warps) per level at 192x64x64, where their bytes take 43 and 31 us; 93 and
+// 79 us while the velocity derivatives held a second cube (96 registers).
 template <typename R, int QH, bool CUM, int PART>
 __global__ void __launch_bounds__(kBlock) k_adjoint_flow(
     const R* __restrict__ muf_next, const R* __restrict__ muh_next, R* __restrict__ muf_out, R* __restrict__ muh_out,
