@@ -317,45 +317,71 @@ __host__ __device__ __forceinline__ constexpr double HALVES(int m, int n, int o)
     return (m == 2 ? 0.5 : 1.0) * (n == 2 ? 0.5 : 1.0) * (o == 2 ? 0.5 : 1.0);
 }
 
-// ---- equilibria as products, for FP64 arithmetic ----------------------------
+// ---- equilibria as products of deviations, for FP64 arithmetic --------------
 // GB300 issues 1.6 FP64 operations per clock and SM, so an FP64 step is bound
 // by their number (about 830 per node update with the equilibria taken through
-// the moment cube: Cumulants-1st at 256x256x1, 20 steps 2.44 ms -> 1.59 ms).
-// The equilibrium of zeroth moment psi at velocity u is psi phi_x phi_y phi_z with phi = (c_s^2 + u^2 +- u)/2
-// and 1 - c_s^2 - u^2 per axis: 12 products for the lines and one operation per
-// population.  Its difference from the reference w ref then carries the
-// rounding of the full population (1e-17 for O(0.1) values), the last place
-// of what FP64 states hold; FP32 arithmetic, whose deviations need the relative
-// precision of the moment form, does not use it.
-template <typename R> struct EqProduct {
-    R xy[9], z[3];  // psi phi_x phi_y by (e_y + 1) * 3 + e_x + 1; phi_z by e_z + 1
-    __device__ __forceinline__ EqProduct(R psi, R ux, R uy, R uz) {
-        R x[3], y[3];
-        axis(ux, x);
-        axis(uy, y);
-        axis(uz, z);
+// the moment cube).  The equilibrium of zeroth moment psi at velocity u is
+// psi phi_x phi_y phi_z with phi = w + d per axis, d = -u^2 at rest and
+// (u^2 +- u)/2 moving.  What is stored is its difference from ref w, taken here
+// axis by axis: a column z differs by C = psi d_z + w_z dpsi, its line y by
+// L = psi phi_z d_y + w_y C and the population by psi phi_y phi_z d_x + w_x L.
+// No full population is formed and taken away again, so a difference keeps its
+// relative precision however small it is, as in the moment cube; and the member
+// at rest of each line, of each column and of the columns is what the other two
+// leave of the total, so that the zeroth moment is the one that went in.
+// Cumulants-1st at 256x256x1, 20 steps: 2.44 ms through the cube -> 1.72 ms, at
+// the cube's accuracy (20 steps of periodic flows against 80 bits: relative
+// error of f 4.6e-16, of h 8.2e-16; the cube 4.2e-16 and 8.4e-16).  As
+// psi phi_x phi_y phi_z - w ref the same takes 1.57 ms, with the rounding of the
+// full population in every difference: 3e-14 to 1e-11 of f, and 1.1e-16 of mass
+// per node and step, always lost.
+template <typename R> struct EqLines {
+    R P[9], L[9];  // line j = (e_y + 1) + 3 (e_z + 1): psi phi_y phi_z, its difference from ref w_y w_z
+    R dp, dm;      // d_x of e_x = +1 and -1
+    __device__ __forceinline__ EqLines(R psi, R dpsi, R ux, R uy, R uz) {
+        R dym, dyp, dzm, dzp, pz[3], C[3];
+        axis(ux, dm, dp);
+        axis(uy, dym, dyp);
+        axis(uz, dzm, dzp);
+        split(psi, psi, dzm, dzp, pz[0], pz[1], pz[2]);
+        split(psi, dpsi, dzm, dzp, C[0], C[1], C[2]);
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const R px = psi * x[i];
-#pragma unroll
-            for (int j = 0; j < 3; ++j) xy[3 * j + i] = px * y[j];
+        for (int z = 0; z < 3; ++z) {
+            split(pz[z], pz[z], dym, dyp, P[3 * z], P[3 * z + 1], P[3 * z + 2]);
+            split(pz[z], C[z], dym, dyp, L[3 * z], L[3 * z + 1], L[3 * z + 2]);
         }
     }
-    static __device__ __forceinline__ void axis(R u, R* t) {
-        const R uu = u * u;
-        t[1] = R(2.0 / 3.0) - uu;
-        t[2] = R(0.5) * (uu + u) + R(1.0 / 6.0);
-        t[0] = t[2] - u;
+    static __device__ __forceinline__ void axis(R u, R& m, R& p) {
+        const R hv = R(0.5) * u;
+        p = hv * u + hv;
+        m = hv * u - hv;
     }
-    // acc + the equilibrium of direction a
-    __device__ __forceinline__ R add(R acc, int a) const { return acc + xy[(EY(a) + 1) * 3 + EX(a) + 1] * z[EZ(a) + 1]; }
+    // the three members of an axis: f d + w t, the one at rest what t leaves
+    static __device__ __forceinline__ void split(R f, R t, R m, R p, R& tm, R& tr, R& tp) {
+        const R w = R(1.0 / 6.0) * t;
+        tp = f * p + w;
+        tm = f * m + w;
+        tr = t - tp - tm;
+    }
+    // the populations of line j
+    __device__ __forceinline__ void line(int j, R& lo, R& mid, R& up) const { split(P[j], L[j], dm, dp, lo, mid, up); }
+    // inv3h of the moments (lo, mid, up), the line's equilibrium added
+    __device__ __forceinline__ void add(int j, R& lo, R& mid, R& up, const InvAxis<R>& k) const {
+        const R t = up + R(1.0 / 6.0) * L[j];
+        const R gp = t + k.p1 * mid + k.p0 * lo + P[j] * dp;
+        const R gm = t + k.m1 * mid + k.m0 * lo + P[j] * dm;
+        mid = lo + L[j] - gp - gm;
+        lo = gm;
+        up = gp;
+    }
 };
 
 // inverse_cube_h of a cube that holds only the non-equilibrium part of the f
 // collision, whose z lines start with one or two moments each (the slots not
-// named in collide_f_force's list are zero and are not read)
+// named in collide_f_force's list are zero and are not read), plus the
+// equilibrium
 template <typename R>
-__device__ __forceinline__ void inverse_cube_neq(R* c, R vx, R vy, R vz) {
+__device__ __forceinline__ void inverse_cube_neq(R* c, R vx, R vy, R vz, const EqLines<R>& eq) {
     const InvAxis<R> kx = inv_axis(vx), ky = inv_axis(vy), kz = inv_axis(vz);
 #pragma unroll
     for (int j = 0; j < 9; ++j) {
@@ -381,7 +407,7 @@ __device__ __forceinline__ void inverse_cube_neq(R* c, R vx, R vy, R vz) {
 #pragma unroll
         for (int x = 0; x < 3; ++x) inv3h<R>(c[9 * z + x], c[9 * z + 3 + x], c[9 * z + 6 + x], ky);
 #pragma unroll
-    for (int j = 0; j < 9; ++j) inv3h<R>(c[3 * j], c[3 * j + 1], c[3 * j + 2], kx);
+    for (int j = 0; j < 9; ++j) eq.add(j, c[3 * j], c[3 * j + 1], c[3 * j + 2], kx);
 }
 
 // ---- parameters -------------------------------------------------------------
@@ -556,13 +582,10 @@ __device__ __forceinline__ void collide_f_force(R* fd, const DevParams& p, const
                 else cb[MIDX(m, n, o)] = neq + drho * Eqh<R>(m, n, o) + rho0 * Dmh<R>(m, n, o, vx, vy, vz, hx, hy, hz);
             }
     if constexpr (std::is_same<R, double>::value) {
-        inverse_cube_neq<R>(cb, vx, vy, vz);
-        const EqProduct<R> eq(rho, vx, vy, vz);
-#pragma unroll
-        for (int a = 0; a < 27; ++a) fd[a] = eq.add(cb[CUBE(a)] - rho0 * R(W27(a)), a);
-        return;
+        inverse_cube_neq<R>(cb, vx, vy, vz, EqLines<R>(rho, drho, vx, vy, vz));
+    } else {
+        inverse_cube_h<R>(cb, vx, vy, vz);
     }
-    inverse_cube_h<R>(cb, vx, vy, vz);
 #pragma unroll
     for (int a = 0; a < 27; ++a) fd[a] = cb[CUBE(a)];
 }
@@ -758,9 +781,11 @@ template <typename R, int QH>
 __device__ __forceinline__ void heq_dev(R* hd, R dpsi, R ux, R uy, R uz, const DevParams& p) {
     const R Tref = par<R>(p.Tref, p.pf.Tref);
     if constexpr (QH == 27 && std::is_same<R, double>::value) {
-        const EqProduct<R> eq(Tref + dpsi, ux, uy, uz);
+        const EqLines<R> eq(Tref + dpsi, dpsi, ux, uy, uz);
 #pragma unroll
-        for (int a = 0; a < 27; ++a) hd[a] = eq.add(-Tref * R(W27(a)), a);
+        for (int j = 0; j < 9; ++j)
+            eq.line(j, hd[DIR(-1, j % 3 - 1, j / 3 - 1)], hd[DIR(0, j % 3 - 1, j / 3 - 1)],
+                    hd[DIR(1, j % 3 - 1, j / 3 - 1)]);
     } else if constexpr (QH == 27) {
         const R tx = ux * ux, ty = uy * uy, tz = uz * uz;
         R cb[27];
