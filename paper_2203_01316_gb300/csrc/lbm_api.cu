@@ -1513,8 +1513,11 @@ lbm_status lbm_step_record_pre(lbm_ctx* c, int n, void* f_rec, void* h_rec) {
     return LBM_OK;
 }
 
+static int flow_acc_parts(const lbm_ctx* c) {
+    return c->p.storage == LBM_F32 ? lbmd::flow_acc_parts<float>() : lbmd::flow_acc_parts<double>();
+}
 static size_t flow_acc_bytes(const lbm_ctx* c) {
-    return 3 * (lbmd::flow_acc_warps(c->N) + (size_t)c->p.ny * c->p.nz) * sizeof(double);
+    return 3 * (lbmd::flow_acc_warps(c->N) * flow_acc_parts(c) + (size_t)c->p.ny * c->p.nz) * sizeof(double);
 }
 
 lbm_status lbm_adjoint_flow_step(lbm_ctx* c, const void* f_level, const void* h_level, const void* muf_next,
@@ -1588,10 +1591,10 @@ lbm_status lbm_adjoint_flow_gradient(lbm_ctx* c, double* dJ_dF, double* dJ_duin,
     if (!c->d_flowacc) return LBM_OK;
     double* out = c->d_scratch + 3 * lbmd::kRedBlocks;  // three results, read back before the next use
     const size_t nw = lbmd::flow_acc_warps(c->N);
-    CK(lbmd::launch_reduce3(c->d_flowacc, (int)nw, c->p.storage == LBM_F32, out, c->d_scratch, c->stream),
-       "flow gradient reduction");
+    const int parts = flow_acc_parts(c);
+    CK(lbmd::launch_reduce3(c->d_flowacc, (int)nw, parts, out, c->d_scratch, c->stream), "flow gradient reduction");
     CK(cudaMemcpyAsync(dJ_dF, out, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "flow gradient copy");
-    CK(lbmd::launch_reduce3(c->d_flowacc + 3 * nw, c->p.ny * c->p.nz, false, out, c->d_scratch, c->stream),
+    CK(lbmd::launch_reduce3(c->d_flowacc + 3 * nw * parts, c->p.ny * c->p.nz, 1, out, c->d_scratch, c->stream),
        "flow gradient reduction");
     CK(cudaMemcpyAsync(dJ_duin, out, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "flow gradient copy");
     if (reset) CK(cudaMemsetAsync(c->d_flowacc, 0, flow_acc_bytes(c), c->stream), "flow gradient reset");

@@ -50,10 +50,10 @@ struct AdjObjective {
 };
 
 constexpr int kBlock = 128;
-// warps of the coupled sweep; its accumulators are [warps][3] for dJ/dF
-// (WideSum, 8 bytes each for either arithmetic), then FP64 [ny nz][3] for dJ/du_in
+// warps of the coupled sweep; its FP64 accumulators are [warps][3][parts] for
+// dJ/dF (parts: FP32 2, FP64 1), then [ny nz][3] for dJ/du_in
 inline size_t flow_acc_warps(int N) { return (size_t)((N + kBlock - 1) / kBlock) * (kBlock / 32); }
-static_assert(sizeof(WideSum<float>) == 8 && sizeof(WideSum<double>) == 8, "one slot size");
+template <typename R> __host__ __device__ constexpr int flow_acc_parts() { return sizeof(R) == 4 ? 2 : 1; }
 constexpr int kRedBlocks = 1216;  // 8 x 152 SMs, partial sums of the reductions
 constexpr int kRedThreads = 256;
 
@@ -77,9 +77,8 @@ constexpr bool step_fills_symmetry(size_t ssize, int qh) { return !(ssize == 2 &
 // symmetry rows: fill them in the post-collision arrays of the current level
 template <typename S, int QH>
 cudaError_t launch_mirror(const Buffers& b, const DevParams& p, cudaStream_t s);
-// out[k] = sum of acc[i * 3 + k] over i < n (the coupled adjoint's accumulators);
-// pairs: acc holds WideSum<float>
-cudaError_t launch_reduce3(const double* acc, int n, bool pairs, double* out, double* scratch, cudaStream_t s);
+// out[k] = sum of acc[(i * 3 + k) * parts + j] over i < n, j < parts (the coupled adjoint's accumulators)
+cudaError_t launch_reduce3(const double* acc, int n, int parts, double* out, double* scratch, cudaStream_t s);
 // out[w] = sum of dlink[l] over the links with lwall[l] == w, for n_walls <=
 // kWallSumMax walls; part: scratch of 3 * kRedBlocks doubles, out after it
 constexpr int kWallSumMax = 64, kWallSumBlocks = 3 * kRedBlocks / kWallSumMax;
@@ -2434,9 +2433,12 @@ __device__ __forceinline__ void adjoint_flow_node(
     }
 }
 
-// accF[warp][3]: accumulators of dJ/dF as WideSum (a warp adds its nodes' terms
-// of a level there), acc_in[row][3]: FP64 accumulators of dJ/du_in per inlet
-// row.  Each slot has one owner, so there are no atomics.  One FP64 slot of six
+// accF[warp][3][parts]: FP64 accumulators of dJ/dF (a warp adds its nodes' terms
+// of a level as a WideSum, and the two parts of that there, since a sweep has any
+// number of levels; a lane for each part, so that the FP64 pipe, 20 clocks per
+// warp instruction, sees a conversion and an addition per level: 4 of them on
+// three lanes took 5 us of 65 a level at 192x64x64), acc_in[row][3]: those of
+// dJ/du_in per inlet row.  Each slot has one owner, so there are no atomics.  One FP64 slot of six
 // per node took 96 B of the f part's 460 B per node, six operations a node on
 // the FP64 pipe, and 1.4 ms to add up at 192x64x64 (60 levels and their
 // recomputation there: 26.30 -> 22.36 ms, with dJ/dQ as WideSum).  Both parts
@@ -2447,7 +2449,7 @@ template <typename R, int QH, bool CUM, int PART>
 __global__ void __launch_bounds__(kBlock) k_adjoint_flow(
     const R* __restrict__ muf_next, const R* __restrict__ muh_next, R* __restrict__ muf_out, R* __restrict__ muh_out,
     const R* __restrict__ gf, const R* __restrict__ gh, const float* __restrict__ theta,
-    double* __restrict__ dtheta, WideSum<R>* __restrict__ accF, double* __restrict__ acc_in, const R* __restrict__ din,
+    double* __restrict__ dtheta, double* __restrict__ accF, double* __restrict__ acc_in, const R* __restrict__ din,
     R* __restrict__ wbuf, const uint8_t* __restrict__ flags, const int32_t* __restrict__ seg_base,
     const uint32_t* __restrict__ wmask, const int32_t* __restrict__ woff, const float* __restrict__ lq,
     const int32_t* __restrict__ lwall, const int32_t* __restrict__ rseg_base, const uint32_t* __restrict__ rmask,
@@ -2474,11 +2476,20 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_flow(
         }
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) v.merge_down(o);
-        if (d < 3 && i == 0) {
-            WideSum<R>* slot = accF + (size_t)((blockIdx.x * kBlock + threadIdx.x) >> 5) * 3 + d;
-            WideSum<R> t = *slot;
-            t.merge(v);
-            *slot = t;
+        constexpr int PARTS = flow_acc_parts<R>();
+        const R hi = __shfl_sync(0xffffffffu, v.hi, lane & 24);
+        R part = hi;
+        if constexpr (PARTS == 2) {
+            const R lo = __shfl_sync(0xffffffffu, v.lo, lane & 24);
+            if (i == 1) part = lo;
+        }
+        if (d < 3 && i < PARTS) {
+            double t = (double)part;
+            if (!isfinite(hi)) {  // beyond the range of the terms: one by one in FP64
+                t = 0.0;
+                for (int k = 0; i == 0 && k < 32; ++k) t += (double)sh[warp][d][k];
+            }
+            accF[((size_t)((blockIdx.x * kBlock + threadIdx.x) >> 5) * 3 + d) * PARTS + i] += t;
         }
     }
 }
@@ -2520,8 +2531,8 @@ cudaError_t launch_adjoint_flow(const Buffers& b, const DevParams& p, const R* f
                                 const R* muf_next, const R* muh_next, R* muf_out, R* muh_out, AdjObjective obj,
                                 double* dtheta, double* acc, const R* din, R* wbuf, cudaStream_t s) {
     const int grid = (p.N + kBlock - 1) / kBlock;
-    WideSum<R>* accF = (WideSum<R>*)acc;
-    double* acc_in = acc + 3 * flow_acc_warps(p.N);
+    double* accF = acc;
+    double* acc_in = acc + 3 * flow_acc_parts<R>() * flow_acc_warps(p.N);
 #define LBM_ADJF_ARGS                                                                                            \
     muf_next, muh_next, muf_out, muh_out, f_level, h_level, b.theta, dtheta, accF, acc_in, din, wbuf, b.flags,  \
         b.seg_base, b.wmask, b.woff, b.lq, b.lwall, b.rseg_base, b.rmask, b.roff, b.rlink, b.dlink, obj, p

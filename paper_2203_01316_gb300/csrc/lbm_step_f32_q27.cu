@@ -56,22 +56,20 @@ cudaError_t launch_stream_map(const Buffers& b, const DevParams& p, int qh, int3
     return cudaGetLastError();
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kRedThreads) k_reduce3(const T* __restrict__ acc, int n, double* __restrict__ part,
-                                                         const RedOut o) {
+__global__ void __launch_bounds__(kRedThreads) k_reduce3(const double* __restrict__ acc, int n, int parts,
+                                                         double* __restrict__ part, const RedOut o) {
     __shared__ double sh[32 * 3];
     double v[3] = {0.0, 0.0, 0.0};
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
 #pragma unroll
-        for (int k = 0; k < 3; ++k) v[k] += acc[(size_t)i * 3 + k].value();
+        for (int k = 0; k < 3; ++k)
+            for (int j = 0; j < parts; ++j) v[k] += acc[((size_t)i * 3 + k) * parts + j];
     if (reduce_in_last_block<3>(v, sh, part, red_counter(part))) write_totals<3>(v, o);
 }
 
-cudaError_t launch_reduce3(const double* acc, int n, bool pairs, double* out, double* scratch, cudaStream_t s) {
+cudaError_t launch_reduce3(const double* acc, int n, int parts, double* out, double* scratch, cudaStream_t s) {
     const int grid = std::min((n + kRedThreads - 1) / kRedThreads, kRedBlocks);
-    const RedOut o{out, nullptr, 0.0, 0};
-    if (pairs) k_reduce3<<<grid, kRedThreads, 0, s>>>((const WideSum<float>*)acc, n, scratch, o);
-    else k_reduce3<<<grid, kRedThreads, 0, s>>>((const WideSum<double>*)acc, n, scratch, o);
+    k_reduce3<<<grid, kRedThreads, 0, s>>>(acc, n, parts, scratch, RedOut{out, nullptr, 0.0, 0});
     return cudaGetLastError();
 }
 

@@ -9,10 +9,13 @@
 namespace lbmd {
 
 // Running sum of R values.  float: Knuth's two-sum keeps the rounding error of
-// every addition (exactly representable) and adds it up beside the sum, so the
-// pair holds the sum to about 2^-48 of its largest partial sum; six FP32
-// additions per value.  An infinity or NaN among the values shows in `hi`, as
-// does a partial sum beyond the float range.  double: one FP64 addition.
+// every addition (exactly representable) and adds it up beside the sum.  The sum
+// of those errors is an FP32 sum itself: after n additions it is off by at most
+// n^2 2^-49 of the largest partial sum (about n 2^-48 for values of either
+// sign), so a pair serves the few dozen values of a node or a warp, and what
+// lasts longer is kept in FP64.  Six FP32 additions per value.  An infinity or
+// NaN among the values shows in `hi`, as does a partial sum beyond the float
+// range.  double: one FP64 addition.
 template <typename R> struct WideSum {
     R hi = R(0);
     __device__ __forceinline__ void add(R x) { hi += x; }
