@@ -909,8 +909,9 @@ cudaError_t launch_balances(const Buffers& b, const DevParams& p, double* scratc
 // after another waited for each link's loads in turn (128x64x64 plate channel:
 // flux 34 us and a reduction of 5 us -> 11 us; 384x128x128 sphere: force 44 us
 // and 5 us -> 25 us; fields, totals, flux and force of that state 764 -> 711 us).
-// Each lane keeps one direction throughout, so the links' values
-// are added as a WideSum and multiplied by the lane's constants once at the end.
+// Each lane keeps one direction throughout, so its constants multiply the sum of
+// its links once at the end.  The sums are FP64: a wall has any number of links,
+// and their values any size.
 constexpr int kWallLanes27 = 32, kWallLanes7 = 8;
 template <int QH> constexpr int wall_lanes() { return QH == 27 ? kWallLanes27 : kWallLanes7; }
 
@@ -1022,14 +1023,13 @@ __global__ void __launch_bounds__(kRedThreads) k_surface_flux(const S* __restric
     using R = typename Acc<S>::R;
     constexpr int L = wall_lanes<QH>();
     __shared__ double sh[32];
-    const size_t N = (size_t)p.N;
     const R Tref = par<R>(p.Tref, p.pf.Tref);
     const int ia = threadIdx.x % L;  // h population of this lane
     const LaneDir d = lane_dir(QH == 27 ? min(ia, 26) : (ia < 4 ? ia : min(ia + 3, 9)));
     const int ib = QH == 27 ? d.b : OPP7(min(ia, 6));
     const R wi = QH == 27 ? (R)d.w : (R)(1.0 / 6.0);
     const R heq2 = R(2) * wi * ((R)Twall[wall] - Tref);
-    WideSum<R> sum;
+    double v[1] = {0.0};
     const int step = gridDim.x * (blockDim.x / L);
     for (int w = blockIdx.x * (blockDim.x / L) + threadIdx.x / L; w < nw; w += step) {
         const uint32_t mask = wmask[w];
@@ -1053,10 +1053,8 @@ __global__ void __launch_bounds__(kRedThreads) k_surface_flux(const S* __restric
             const R hb_b = ld<R>(pop<S, QH>(hA, ib, p.N, n));
             hin = (-ha_b + (R(2) * qq - R(1)) * hb_b + heq2) / (R(2) * qq);
         }
-        sum.add(hin);
-        sum.add(-ha_b);
+        v[0] += (double)hin - (double)ha_b;
     }
-    double v[1] = {sum.value()};
     if (reduce_in_last_block<1>(v, sh, part, red_counter(part))) write_totals<1>(v, o);
 }
 
@@ -1089,10 +1087,9 @@ __global__ void __launch_bounds__(kRedThreads) k_wall_force(const S* __restrict_
     using R = typename Acc<S>::R;
     constexpr int L = kWallLanes27;
     __shared__ double sh[3 * 32];
-    const size_t N = (size_t)p.N;
     const int ia = threadIdx.x % L;
     const LaneDir d = lane_dir(min(ia, 26));
-    WideSum<R> sum;
+    double sum = 0.0;
     int links = 0;
     const int step = gridDim.x * (blockDim.x / L);
     for (int w = blockIdx.x * (blockDim.x / L) + threadIdx.x / L; w < nw; w += step) {
@@ -1113,11 +1110,10 @@ __global__ void __launch_bounds__(kRedThreads) k_wall_force(const S* __restrict_
             const R qq = (R)fmaxf(q, 0.5f);
             fin = (fa_b + (R(2) * qq - R(1)) * ld<R>(pop<S, QH>(fA, d.b, p.N, n))) / (R(2) * qq);
         }
-        sum.add(fa_b);
-        sum.add(fin);
+        sum += (double)fa_b + (double)fin;
         ++links;
     }
-    const double carried = sum.value() + 2.0 * d.w * p.rho0 * (double)links;
+    const double carried = sum + 2.0 * d.w * p.rho0 * (double)links;
     double v[3] = {d.ex * carried, d.ey * carried, d.ez * carried};
     if (reduce_in_last_block<3>(v, sh, part, red_counter(part))) write_totals<3>(v, o);
 }
