@@ -11,6 +11,7 @@
 
 #include "../../include/lbm.h"
 #include "lbm_kernels.cuh"
+#include "lbm_reach.h"
 
 using lbmd::Acc;
 using lbmd::Buffers;
@@ -298,6 +299,14 @@ template <typename T> lbm_status to_host(lbm_ctx* c, const T* src, size_t count,
 
 }  // namespace
 
+// whether kernels of this context may access the caller's buffer p themselves
+static bool own_memory(const lbm_ctx* c, const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) == cudaSuccess) return lbmd::kernel_reaches(a, c->device);
+    cudaGetLastError();
+    return false;
+}
+
 // paired storage <-> the state format ([27][N] f, then [27][N] h); count = 27 N
 __global__ void k_unpair(const uint32_t* __restrict__ w, unsigned short* __restrict__ f, unsigned short* __restrict__ h,
                          uint32_t count) {
@@ -314,7 +323,7 @@ __global__ void k_pair(const unsigned short* __restrict__ f, const unsigned shor
 }
 
 // The paired state of the current level to (save) or from `buf` in the state
-// format.  Host memory, and device memory at an odd address, go through the
+// format.  Memory that kernels cannot access, or at an odd address, goes through the
 // array of the other level, which holds nothing that is still needed but the
 // zeros at its solid nodes (cleared again).
 static cudaError_t copy_paired(lbm_ctx* c, char* buf, bool is_device, bool save) {
@@ -322,7 +331,7 @@ static cudaError_t copy_paired(lbm_ctx* c, char* buf, bool is_device, bool save)
     const size_t half = (size_t)count * 2;
     uint32_t* words = (uint32_t*)c->f[c->cur_f];
     char* other = (char*)c->f[1 - c->cur_f];
-    const bool direct = is_device && ((uintptr_t)buf & 1) == 0;
+    const bool direct = is_device && ((uintptr_t)buf & 1) == 0 && own_memory(c, buf);
     char* flat = direct ? buf : other;
     const unsigned grid = (count + 255) / 256;
     cudaError_t e = cudaSuccess;
@@ -1273,7 +1282,7 @@ lbm_status lbm_save_state(lbm_ctx* c, void* host_buf, size_t* bytes, int is_devi
     hd.hbytes = (uint64_t)c->qh * c->N * c->ssize;
     char* out = (char*)host_buf;
     const cudaMemcpyKind kind = is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    if (is_device && !paired(c) && need <= kSmallState && ((uintptr_t)out & 7) == 0) {
+    if (is_device && !paired(c) && need <= kSmallState && ((uintptr_t)out & 7) == 0 && own_memory(c, out)) {
         const uint32_t nf = (uint32_t)27 * c->N, nh = (uint32_t)c->qh * c->N;
         const unsigned grid = std::min<uint32_t>((nf + nh + 255) / 256, 152 * 8);
         const void *f = c->f[c->cur_f], *h = c->h[c->cur_h];
