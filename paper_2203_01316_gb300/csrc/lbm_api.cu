@@ -307,52 +307,177 @@ static bool own_memory(const lbm_ctx* c, const void* p) {
     return false;
 }
 
-// paired storage <-> the state format ([27][N] f, then [27][N] h); count = 27 N
-__global__ void k_unpair(const uint32_t* __restrict__ w, unsigned short* __restrict__ f, unsigned short* __restrict__ h,
-                         uint32_t count) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count) return;
-    const uint32_t v = w[i];
-    f[i] = (unsigned short)(v & 0xffffu);
-    h[i] = (unsigned short)(v >> 16);
+// ---- paired storage <-> the state format ([27][N] f, then [27][N] h) --------
+// A block takes kPairTile words through shared memory: four words per access on
+// the side of the state, four halves on the other, whose two arrays start on any
+// even address (the h part behind 27 N halves); the ends that do not fill eight
+// bytes go one by one.  Bound by the bytes, 27 x 8 per node: 384x128x128, 1.36 GB,
+// 216 us to save and 227 us to load (two cudaMemcpyAsync of separate arrays: 234
+// and 232 us; one word and two halves per thread: 471 and 517 us).
+constexpr int kPairTile = 2048, kPairThreads = 256;
+
+constexpr int kPairVecs = kPairTile / 4 / kPairThreads;  // accesses of a thread to a tile
+
+// m halves at p as `body` groups of four on eight-byte boundaries behind `head`
+struct Halves {
+    int head, body;
+    __device__ __forceinline__ Halves(const unsigned short* p, int m)
+        : head(min(m, (int)((8 - ((uintptr_t)p & 7)) & 7) >> 1)), body((m - head) >> 2) {}
+    // those outside the groups: their index, of m - 4 body
+    __device__ __forceinline__ int end(int i) const { return i < head ? i : 4 * body + i; }
+};
+__device__ __forceinline__ void store_halves(unsigned short* __restrict__ p, const unsigned short* s, int m) {
+    const Halves a(p, m);
+#pragma unroll
+    for (int j = 0; j < kPairVecs; ++j) {
+        const int i = threadIdx.x + j * kPairThreads;
+        const unsigned short* t = s + a.head + 4 * i;
+        if (i < a.body) *(ushort4*)(p + a.head + 4 * i) = make_ushort4(t[0], t[1], t[2], t[3]);
+    }
+    const int i = threadIdx.x;
+    if (i < m - 4 * a.body) p[a.end(i)] = s[a.end(i)];
 }
-__global__ void k_pair(const unsigned short* __restrict__ f, const unsigned short* __restrict__ h,
-                       uint32_t* __restrict__ w, uint32_t count) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) w[i] = (uint32_t)f[i] | (uint32_t)h[i] << 16;
+// words w (16-byte aligned) -> f, h
+__global__ void __launch_bounds__(kPairThreads) k_unpair(const uint32_t* __restrict__ w, unsigned short* __restrict__ f,
+                                                         unsigned short* __restrict__ h, uint32_t count) {
+    __shared__ __align__(8) unsigned short sf[kPairTile], sh[kPairTile];
+    const uint32_t base = blockIdx.x * kPairTile;
+    const int m = (int)min((uint32_t)kPairTile, count - base);
+    uint4 v[kPairVecs];
+#pragma unroll
+    for (int j = 0; j < kPairVecs; ++j) {
+        const int i = threadIdx.x + j * kPairThreads;
+        if (i < m / 4) v[j] = ((const uint4*)(w + base))[i];
+    }
+#pragma unroll
+    for (int j = 0; j < kPairVecs; ++j) {
+        const int i = threadIdx.x + j * kPairThreads;
+        if (i >= m / 4) break;
+        *(uint2*)(sf + 4 * i) = make_uint2(__byte_perm(v[j].x, v[j].y, 0x5410), __byte_perm(v[j].z, v[j].w, 0x5410));
+        *(uint2*)(sh + 4 * i) = make_uint2(__byte_perm(v[j].x, v[j].y, 0x7632), __byte_perm(v[j].z, v[j].w, 0x7632));
+    }
+    if ((int)threadIdx.x < (m & 3)) {
+        const int i = (m & ~3) + threadIdx.x;
+        sf[i] = (unsigned short)(w[base + i] & 0xffffu);
+        sh[i] = (unsigned short)(w[base + i] >> 16);
+    }
+    __syncthreads();
+    store_halves(f + base, sf, m);
+    store_halves(h + base, sh, m);
+}
+// f, h -> words w
+__global__ void __launch_bounds__(kPairThreads) k_pair(const unsigned short* __restrict__ f,
+                                                       const unsigned short* __restrict__ h, uint32_t* __restrict__ w,
+                                                       uint32_t count) {
+    __shared__ __align__(8) unsigned short sf[kPairTile], sh[kPairTile];
+    const uint32_t base = blockIdx.x * kPairTile;
+    const int m = (int)min((uint32_t)kPairTile, count - base);
+    const Halves a(f + base, m), b(h + base, m);
+    ushort4 u[kPairVecs], v[kPairVecs];  // all loads before the first store
+#pragma unroll
+    for (int j = 0; j < kPairVecs; ++j) {
+        const int i = threadIdx.x + j * kPairThreads;
+        if (i < a.body) u[j] = *(const ushort4*)(f + base + a.head + 4 * i);
+        if (i < b.body) v[j] = *(const ushort4*)(h + base + b.head + 4 * i);
+    }
+#pragma unroll
+    for (int j = 0; j < kPairVecs; ++j) {
+        const int i = threadIdx.x + j * kPairThreads;
+        unsigned short *s = sf + a.head + 4 * i, *t = sh + b.head + 4 * i;
+        if (i < a.body) s[0] = u[j].x, s[1] = u[j].y, s[2] = u[j].z, s[3] = u[j].w;
+        if (i < b.body) t[0] = v[j].x, t[1] = v[j].y, t[2] = v[j].z, t[3] = v[j].w;
+    }
+    if ((int)threadIdx.x < m - 4 * a.body) sf[a.end(threadIdx.x)] = f[base + a.end(threadIdx.x)];
+    if ((int)threadIdx.x < m - 4 * b.body) sh[b.end(threadIdx.x)] = h[base + b.end(threadIdx.x)];
+    __syncthreads();
+    for (int i = threadIdx.x; i < m / 4; i += kPairThreads) {
+        const uint2 x = *(const uint2*)(sf + 4 * i), y = *(const uint2*)(sh + 4 * i);
+        ((uint4*)(w + base))[i] = make_uint4(__byte_perm(x.x, y.x, 0x5410), __byte_perm(x.x, y.x, 0x7632),
+                                             __byte_perm(x.y, y.y, 0x5410), __byte_perm(x.y, y.y, 0x7632));
+    }
+    if ((int)threadIdx.x < (m & 3)) {
+        const int i = (m & ~3) + threadIdx.x;
+        w[base + i] = (uint32_t)sf[i] | (uint32_t)sh[i] << 16;
+    }
+}
+// zeros at the solid nodes of a paired level that served as scratch memory
+__global__ void k_clear_solid(uint32_t* __restrict__ w, const uint8_t* __restrict__ flags, int N) {
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= N || (flags[n] & 3) != lbmd::T_SOLID) return;
+    for (int a = 0; a < 27; ++a) w[(uint32_t)a * (uint32_t)N + (uint32_t)n] = 0u;
+}
+static cudaError_t clear_solid(lbm_ctx* c, void* level) {
+    k_clear_solid<<<(c->N + 255) / 256, 256, 0, c->stream>>>((uint32_t*)level, c->d_flags, c->N);
+    return cudaGetLastError();
+}
+
+// the context's second stream and its events, made at first use
+static bool side_stream(lbm_ctx* c) {
+    if (!c->side && cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess) c->side = nullptr;
+    if (!c->fork && cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess) c->fork = nullptr;
+    if (!c->join && cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming) != cudaSuccess) c->join = nullptr;
+    if (c->side && c->fork && c->join) return true;
+    cudaGetLastError();
+    return false;
+}
+// work queued on b from here on waits for what a holds now
+static cudaError_t wait_for(cudaStream_t b, cudaStream_t a, cudaEvent_t ev) {
+    if (a == b) return cudaSuccess;
+    const cudaError_t e = cudaEventRecord(ev, a);
+    return e == cudaSuccess ? cudaStreamWaitEvent(b, ev, 0) : e;
 }
 
 // The paired state of the current level to (save) or from `buf` in the state
-// format.  Memory that kernels cannot access, or at an odd address, goes through the
-// array of the other level, which holds nothing that is still needed but the
-// zeros at its solid nodes (cleared again).
+// format.  Memory that kernels cannot access, or at an odd address, goes through
+// the array of the other level, which holds nothing that is still needed but the
+// zeros at its solid nodes (cleared again).  An eighth is converted before or
+// after the copies, which take longer than the rest of the conversion.
 static cudaError_t copy_paired(lbm_ctx* c, char* buf, bool is_device, bool save) {
     const uint32_t count = 27u * (uint32_t)c->N;
     const size_t half = (size_t)count * 2;
     uint32_t* words = (uint32_t*)c->f[c->cur_f];
     char* other = (char*)c->f[1 - c->cur_f];
     const bool direct = is_device && ((uintptr_t)buf & 1) == 0 && own_memory(c, buf);
-    char* flat = direct ? buf : other;
-    const unsigned grid = (count + 255) / 256;
-    cudaError_t e = cudaSuccess;
+    auto convert = [&](char* flat, uint32_t lo, uint32_t m) {
+        const unsigned grid = (m + kPairTile - 1) / kPairTile;
+        unsigned short *f = (unsigned short*)flat + lo, *h = (unsigned short*)(flat + half) + lo;
+        if (save) k_unpair<<<grid, kPairThreads, 0, c->stream>>>(words + lo, f, h, m);
+        else k_pair<<<grid, kPairThreads, 0, c->stream>>>(f, h, words + lo, m);
+        return cudaGetLastError();
+    };
+    if (direct) return convert(buf, 0, count);
+    const cudaStream_t side = side_stream(c) ? c->side : c->stream;
+    const cudaMemcpyKind kind =
+        is_device ? cudaMemcpyDeviceToDevice : (save ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice);
+    auto copy = [&](size_t at, size_t halves) {
+        if (halves == 0) return cudaSuccess;
+        return cudaMemcpyAsync(save ? buf + at : other + at, save ? other + at : buf + at, halves * 2, kind, side);
+    };
+    const uint32_t cut = (save ? count / 8 : count - count / 8) / kPairTile * kPairTile;
+    cudaError_t e = wait_for(side, c->stream, c->fork);  // the other level is free from here on
+    auto then = [&](auto f) {
+        if (e == cudaSuccess) e = f();
+    };
     if (save) {
-        k_unpair<<<grid, 256, 0, c->stream>>>(words, (unsigned short*)flat, (unsigned short*)(flat + half), count);
-        e = cudaGetLastError();
-        if (!direct && e == cudaSuccess)
-            e = cudaMemcpyAsync(buf, flat, 2 * half, is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                                c->stream);
+        if (cut) then([&] { return convert(other, 0, cut); });
+        then([&] { return wait_for(side, c->stream, c->fork); });
+        then([&] { return copy(0, cut); });
+        then([&] { return convert(other, cut, count - cut); });
+        then([&] { return wait_for(side, c->stream, c->fork); });
+        then([&] { return copy((size_t)cut * 2, count - cut); });
+        then([&] { return copy(half, count); });
     } else {
-        if (!direct)
-            e = cudaMemcpyAsync(flat, buf, 2 * half, is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                                c->stream);
-        if (e == cudaSuccess) {
-            k_pair<<<grid, 256, 0, c->stream>>>((const unsigned short*)flat, (const unsigned short*)(flat + half), words,
-                                                count);
-            e = cudaGetLastError();
-        }
+        then([&] { return copy(0, count); });
+        then([&] { return copy(half, cut); });
+        then([&] { return wait_for(c->stream, side, c->join); });
+        if (cut) then([&] { return convert(other, 0, cut); });
+        then([&] { return copy(half + (size_t)cut * 2, count - cut); });
+        then([&] { return wait_for(c->stream, side, c->join); });
+        then([&] { return convert(other, cut, count - cut); });
     }
-    if (!direct && e == cudaSuccess) e = cudaMemsetAsync(other, 0, 2 * half, c->stream);
-    return e;
+    const cudaError_t j = wait_for(c->stream, side, c->join);
+    if (e == cudaSuccess) e = j;
+    return e == cudaSuccess ? clear_solid(c, other) : e;
 }
 
 struct StateHeader {
@@ -1020,16 +1145,11 @@ static lbm_status step_once(lbm_ctx* c, int level = 0, bool forked = false) {
     return LBM_OK;
 }
 
-// whether captured steps have a side branch (its stream and events made at
-// first use; without them the launches stay in one line)
+// whether captured steps have a side branch (without the second stream the
+// launches stay in one line)
 static bool side_branch(lbm_ctx* c) {
     if (!c->dp.zou_he && !(c->ssize == 2 && c->dp.nwall > 0)) return false;
-    if (!c->side && cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess) c->side = nullptr;
-    if (!c->fork && cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess) c->fork = nullptr;
-    if (!c->join && cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming) != cudaSuccess) c->join = nullptr;
-    if (c->side && c->fork && c->join) return true;
-    cudaGetLastError();
-    return false;
+    return side_stream(c);
 }
 
 // A graph of two plain steps for the current buffers and parameters
@@ -1303,6 +1423,9 @@ lbm_status lbm_save_state(lbm_ctx* c, void* host_buf, size_t* bytes, int is_devi
         std::memcpy(out, &hd, sizeof(hd));
     }
     if (paired(c)) {
+        // the rows as the step after this state reads them: copy_paired leaves
+        // none of their former values in the level that the next step writes
+        CK(fill_mirror(c, buffers(c)), "symmetry rows launch");
         CK(copy_paired(c, out + sizeof(hd), is_device != 0, true), "state copy");
     } else {
         CK(cudaMemcpyAsync(out + sizeof(hd), c->f[c->cur_f], hd.fbytes, kind, c->stream), "state copy");
