@@ -1093,8 +1093,8 @@ static cudaError_t fill_mirror(lbm_ctx* c, const Buffers& b) {
 // before the first step of a call (the state may come from lbm_init_fields or
 // lbm_load_state) where the steps then keep the rows; launch_level fills them
 // for each step otherwise
-static lbm_status fill_mirror_once(lbm_ctx* c) {
-    if (!lbmd::step_fills_symmetry(c->ssize, c->qh)) return LBM_OK;
+static lbm_status fill_mirror_once(lbm_ctx* c, bool advance_h, bool rec) {
+    if (!lbmd::step_fills_symmetry(c->ssize, c->qh, advance_h, rec)) return LBM_OK;
     const cudaError_t e = fill_mirror(c, buffers(c));
     return e == cudaSuccess ? LBM_OK : cuda_fail(c, e, "symmetry rows launch");
 }
@@ -1102,7 +1102,8 @@ static lbm_status fill_mirror_once(lbm_ctx* c) {
 // the launches of one step: the step's own and the Zou-He inlet.  forked (in
 // a graph capture): the inlet and the wall nodes' launch go to the side branch
 static cudaError_t launch_level(lbm_ctx* c, const Buffers& b, const DevParams& p, bool advance_h, bool forked = false) {
-    cudaError_t e = lbmd::step_fills_symmetry(c->ssize, c->qh) ? cudaSuccess : fill_mirror(c, b);
+    const bool kept = lbmd::step_fills_symmetry(c->ssize, c->qh, advance_h, b.urec != nullptr);
+    cudaError_t e = kept ? cudaSuccess : fill_mirror(c, b);
     if (e != cudaSuccess) return e;
     const cudaStream_t side = forked ? c->side : c->stream;
     if (forked) {
@@ -1215,7 +1216,7 @@ lbm_status lbm_step(lbm_ctx* c, int n) {
     if (!c->initialised) return fail(c, LBM_ERR_STATE, "initialise the fields first");
     DeviceGuard g(c->device);
     if (n > 0) {
-        const lbm_status st = fill_mirror_once(c);
+        const lbm_status st = fill_mirror_once(c, true, false);
         if (st != LBM_OK) return st;
     }
     // launch-bound stretches replay graphs of two steps (LBM_STEP_AUTO)
@@ -1532,7 +1533,7 @@ lbm_status lbm_step_record(lbm_ctx* c, int n, void* u_rec, int advance_h) {
     if (!c->initialised) return fail(c, LBM_ERR_STATE, "initialise the fields first");
     DeviceGuard g(c->device);
     const size_t rsize = c->p.storage == LBM_F64 ? sizeof(double) : sizeof(float);
-    lbm_status st = n > 0 ? fill_mirror_once(c) : LBM_OK;
+    lbm_status st = n > 0 ? fill_mirror_once(c, advance_h != 0, true) : LBM_OK;
     if (st != LBM_OK) return st;
     for (int i = 0; i < n; ++i) {
         Buffers b = buffers(c);
@@ -1629,7 +1630,7 @@ lbm_status lbm_step_record_pre(lbm_ctx* c, int n, void* f_rec, void* h_rec) {
         return fail(c, LBM_ERR_INVALID, "pre-collision records need FP32 or FP64 storage");
     DeviceGuard g(c->device);
     const size_t rsize = c->ssize;
-    lbm_status st = n > 0 ? fill_mirror_once(c) : LBM_OK;
+    lbm_status st = n > 0 ? fill_mirror_once(c, true, false) : LBM_OK;
     if (st != LBM_OK) return st;
     for (int i = 0; i < n; ++i) {
         Buffers b = buffers(c);

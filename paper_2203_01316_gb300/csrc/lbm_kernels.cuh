@@ -73,7 +73,10 @@ cudaError_t launch_adjoint(const Buffers& b, const DevParams& p, const R* u_leve
 template <typename S, int QH>
 cudaError_t launch_inlet(const Buffers& b, const DevParams& p, cudaStream_t s, bool advance_h);
 // whether a step leaves the symmetry rows of the level that it writes filled
-constexpr bool step_fills_symmetry(size_t ssize, int qh) { return !(ssize == 2 && qh == 27); }
+// (store_symmetry_rows); rec: it records u
+constexpr bool step_fills_symmetry(size_t ssize, int qh, bool do_h, bool rec) {
+    return do_h ? ssize >= 4 && !rec : !(ssize == 2 && qh == 27);
+}
 // symmetry rows: fill them in the post-collision arrays of the current level
 template <typename S, int QH>
 cudaError_t launch_mirror(const Buffers& b, const DevParams& p, cudaStream_t s);
@@ -327,16 +330,17 @@ template <typename R> __device__ __forceinline__ R wdiv(R a, R b) {
 // links).  The threads of the neighbour rows write it with their own node, so
 // that no launch has to fill it before the next step (confined cylinder
 // 1000x152: k_mirror took 26.6 us and k_inlet 10.1 us of 45 us per step; 24 us
-// now).  Reads back the node's own
-// stores, which holds the rounded 16-bit values too.
+// now).  Reads back the node's own stores.
 // Three rolled groups of nine populations, so that the rest of the step keeps
-// its registers.  The 16-bit D3Q27 step, which has none to spare, stays without
-// it (0.9% slower on every grid) and has the rows filled before each step.
+// its registers.  Two kinds of step stay without it and have the rows filled
+// before each step, since it slowed them on every grid: steps of f and h in
+// 16-bit storage (0.9% for either lattice) and those that record u (FP32: 48 B
+// of spill for 16, 1.2%).
 static __constant__ unsigned char kFlipY[27] = {
     FLIPY(0),  FLIPY(1),  FLIPY(2),  FLIPY(3),  FLIPY(4),  FLIPY(5),  FLIPY(6),  FLIPY(7),  FLIPY(8),
     FLIPY(9),  FLIPY(10), FLIPY(11), FLIPY(12), FLIPY(13), FLIPY(14), FLIPY(15), FLIPY(16), FLIPY(17),
     FLIPY(18), FLIPY(19), FLIPY(20), FLIPY(21), FLIPY(22), FLIPY(23), FLIPY(24), FLIPY(25), FLIPY(26)};
-template <typename S, int Q, uint32_t P>  // P: elements per population of a node
+template <typename S, int Q, uint32_t P = 1>  // P: elements per population of a node
 __device__ __forceinline__ void copy_flipped(S* X, int from, int to, int N) {
     constexpr int G = Q == 27 ? 9 : 7;
 #pragma unroll 1
@@ -348,7 +352,7 @@ __device__ __forceinline__ void copy_flipped(S* X, int from, int to, int N) {
         for (int k = 0; k < G; ++k) X[P * soa(Q == 27 ? (int)kFlipY[i + k] : HFLIPY<7>(k), N, to)] = v[k];
     }
 }
-template <typename S, int QH, bool DO_H>
+template <typename S, int QH, bool DO_H, uint32_t P = 1>
 __device__ __forceinline__ void store_symmetry_rows(S* fB, S* hB, int n, const DevParams& p) {
     if (!(p.mirror_lo | p.mirror_hi)) return;
     int x, y, z;
@@ -357,8 +361,8 @@ __device__ __forceinline__ void store_symmetry_rows(S* fB, S* hB, int n, const D
     for (int side = 0; side < 2; ++side) {
         if (side == 0 ? !(p.mirror_lo && y == 1) : !(p.mirror_hi && y == p.ny - 2)) continue;
         const int g = side == 0 ? n - p.nx : n + p.nx;
-        copy_flipped<S, 27, paired<S, QH>() ? 2u : 1u>(fB, n, g, p.N);
-        if constexpr (DO_H) copy_flipped<S, QH, paired<S, QH>() ? 2u : 1u>(hB, n, g, p.N);
+        copy_flipped<S, 27, P>(fB, n, g, p.N);
+        if constexpr (DO_H) copy_flipped<S, QH>(hB, n, g, p.N);
     }
 }
 
@@ -443,7 +447,8 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
             urec[N + n] = par<R>(p.uin[1], p.pf.uin[1]);
             urec[2 * N + n] = par<R>(p.uin[2], p.pf.uin[2]);
         }
-        if constexpr (WM != 2 && step_fills_symmetry(sizeof(S), QH)) store_symmetry_rows<S, QH, DO_H || paired<S, QH>()>(fB, hB, n, p);
+        if constexpr (step_fills_symmetry(sizeof(S), QH, DO_H, REC))
+            store_symmetry_rows<S, QH, DO_H>(fB, hB, n, p);
         return;
     }
     uint32_t mask = 0;
@@ -596,7 +601,7 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
     }
     collide_store_h<S, QH, CUM, TRT>(hd, fB, hB, n, p, ux, uy, uz, Q, rs, fc);
     }
-    if constexpr (WM != 2 && step_fills_symmetry(sizeof(S), QH)) store_symmetry_rows<S, QH, DO_H || paired<S, QH>()>(fB, hB, n, p);
+    if constexpr (step_fills_symmetry(sizeof(S), QH, DO_H, REC)) store_symmetry_rows<S, QH, DO_H>(fB, hB, n, p);
 }
 
 // With many wall nodes the plain 16-bit step runs as two launches: every
@@ -1638,7 +1643,7 @@ __global__ void __launch_bounds__(kBlock) k_inlet(const S* __restrict__ fA, S* _
         const R Q = theta ? (R)__ldg(theta + n) : R(0);
         collide_store_h<S, QH, CUM>(hd, fB, hB, n, p, vx, vy, vz, Q, rs, fc);
     }
-    if constexpr (step_fills_symmetry(sizeof(S), QH)) store_symmetry_rows<S, QH, DO_H || paired<S, QH>()>(fB, hB, n, p);
+    if constexpr (step_fills_symmetry(sizeof(S), QH, DO_H, false)) store_symmetry_rows<S, QH, DO_H>(fB, hB, n, p);
 }
 
 template <typename S, int QH>
@@ -1655,9 +1660,9 @@ cudaError_t launch_inlet(const Buffers& b, const DevParams& p, cudaStream_t s, b
     return cudaGetLastError();
 }
 
-// The symmetry rows of the current level, filled before the first step of a
-// call (after that each step keeps them, store_symmetry_rows): 27 + Q_h values
-// per thread, all loaded before any is stored
+// The symmetry rows of the current level, filled before the first step of a call
+// where the steps then keep them (step_fills_symmetry) and before each step
+// elsewhere: 27 + Q_h values per thread, all loaded before any is stored
 template <typename S, int QH>
 __global__ void k_mirror(S* __restrict__ fA, S* __restrict__ hA, const DevParams p) {
     const int per = p.nx * p.nz;
