@@ -1526,12 +1526,50 @@ static lbm_status check_objective(lbm_ctx* c, const lbm_objective* o) {
     return LBM_OK;
 }
 
+// Two or more f-only steps of paired storage.  Words would move h along at every
+// step (216 B per node beside a second load of the node's own words: 293 us a
+// step at 384x128x128 FP16, where f alone takes 197 us), so f leaves the words
+// with the first step, alternates between two arrays of its own in the level
+// that the next step writes, and goes back into the words with the last; h stays.
+// The level of the state remains the current one.  Ten steps: 2929 -> 2070 us
+// (1996 us with f and h always apart: the first and the last step touch words).
+// One step alone keeps the words: apart, it would have to read and write them too.
+static lbm_status record_f_apart(lbm_ctx* c, int n, char* u_rec) {
+    char *level = (char*)c->f[c->cur_f], *other = (char*)c->f[1 - c->cur_f];
+    char* own[2] = {other, other + (size_t)27 * c->N * c->ssize};
+    for (int i = 0; i < n; ++i) {
+        Buffers b = buffers(c);
+        if (i == 0) CK(fill_mirror(c, b), "symmetry rows launch");
+        c->dp.step += 1;
+        const DevParams p = c->dp;
+        b.fA = i == 0 ? level : own[(i - 1) & 1];
+        b.fB = i == n - 1 ? level : own[i & 1];
+        b.f_words = i == 0 ? 1 : (i == n - 1 ? 2 : 0);
+        b.hA = b.hB = nullptr;
+        b.urec = u_rec + (size_t)i * 3 * c->N * sizeof(float);
+        const cudaError_t e = dispatch(c, [&](auto tag) {
+            using S = typename decltype(tag)::S;
+            if constexpr (sizeof(S) == 2) {  // with its h apart, f is stored as beside D3Q7 h
+                cudaError_t r = lbmd::launch_step<S, 7>(b, p, c->stream, false, c->stream);
+                if (r == cudaSuccess && p.zou_he) r = lbmd::launch_inlet<S, 7>(b, p, c->stream, false);
+                return r;
+            } else {
+                return cudaErrorInvalidValue;
+            }
+        });
+        if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
+    }
+    CK(clear_solid(c, other), "f-only steps");
+    return LBM_OK;
+}
+
 lbm_status lbm_step_record(lbm_ctx* c, int n, void* u_rec, int advance_h) {
     if (!c) return LBM_ERR_INVALID;
     if (n < 0) return fail(c, LBM_ERR_INVALID, "n must be >= 0");
     if (n > 0 && !u_rec) return fail(c, LBM_ERR_INVALID, "null velocity record");
     if (!c->initialised) return fail(c, LBM_ERR_STATE, "initialise the fields first");
     DeviceGuard g(c->device);
+    if (paired(c) && !advance_h && n >= 2) return record_f_apart(c, n, (char*)u_rec);
     const size_t rsize = c->p.storage == LBM_F64 ? sizeof(double) : sizeof(float);
     lbm_status st = n > 0 ? fill_mirror_once(c, advance_h != 0, true) : LBM_OK;
     if (st != LBM_OK) return st;

@@ -28,6 +28,8 @@ struct Buffers {
     const int32_t* lwall;     // per link wall id
     const float* Twall;       // per wall temperature
     int nw;                   // number of wall nodes
+    int f_words;              // f-only steps of 16-bit storage: 1 fA, 2 fB holds f as the low halves of
+                              // (f, h) words, the other one (0: both) as an array of its own
     // adjoint: nodes y that are x_f = x - e_a of a link (x, a) with q <= 1/2
     const int32_t* rseg_base; // such nodes before each 32-node segment
     const uint32_t* rmask;    // bit a set: y + e_a has link a with q <= 1/2
@@ -196,6 +198,7 @@ __device__ __forceinline__ uint32_t soa(int i, int N, int node) {
 // half the bytes per instruction and L1 cycle: FP16 384x128x128,
 // ten steps and a copy: 4.21 -> 3.79 ms, the same bits
 template <typename S, int QH> constexpr bool paired() { return sizeof(S) == 2 && QH == 27; }
+// (lbm_step_record without h works on separate f arrays meanwhile; see there)
 // address of population i of a node in the f or h array X of a state
 template <typename S, int QH, typename P> __device__ __forceinline__ P* pop(P* X, int i, int N, int node) {
     return X + (paired<S, QH>() ? 2u : 1u) * soa(i, N, node);
@@ -234,12 +237,12 @@ __device__ __forceinline__ void round16(const float* v, uint32_t* c, SrStream& r
     if (p.stochastic) round16<true, S, Q>(v, c, rs);
     else round16<false, S, Q>(v, c, rs);
 }
-// c (from round16) of node n into X[i * N + n]
-template <typename S, int Q>
+// c (from round16) of node n into X[P (i * N + n)]
+template <typename S, int Q, uint32_t P = 1>
 __device__ __forceinline__ void store16(S* __restrict__ X, const uint32_t* c, int n, int N) {
 #pragma unroll
     for (int i = 0; i < Q; ++i)
-        *(unsigned short*)(X + soa(i, N, n)) = (unsigned short)((i & 1) ? c[i / 2] >> 16 : c[i / 2] & 0xffffu);
+        *(unsigned short*)(X + P * soa(i, N, n)) = (unsigned short)((i & 1) ? c[i / 2] >> 16 : c[i / 2] & 0xffffu);
 }
 // the words (f_i, h_i) of node n from the rounded f and h
 template <typename S>
@@ -254,8 +257,9 @@ struct Rounded27 {
     uint32_t c[14];
 };
 
-// fc: paired storage keeps the rounded values there until h is known
-template <typename S, int QH>
+// fc: paired storage keeps the rounded values there until h is known; P:
+// elements per population of fB (16-bit storage)
+template <typename S, int QH, uint32_t P = 1>
 __device__ __forceinline__ void collide_store_f(typename Acc<S>::R* fd, S* __restrict__ fB, int n,
                                                 const DevParams& p, typename Acc<S>::R& ux,
                                                 typename Acc<S>::R& uy, typename Acc<S>::R& uz, SrStream& rs,
@@ -265,7 +269,7 @@ __device__ __forceinline__ void collide_store_f(typename Acc<S>::R* fd, S* __res
     collide_f<R>(fd, p, ux, uy, uz, rho);
     if constexpr (sizeof(S) == 2) {
         round16<S, 27>(fd, fc.c, rs, p);
-        if constexpr (!paired<S, QH>()) store16<S, 27>(fB, fc.c, n, p.N);
+        if constexpr (!paired<S, QH>()) store16<S, 27, P>(fB, fc.c, n, p.N);
     } else {
 #pragma unroll
         for (int a = 0; a < 27; ++a) st(fB + soa(a, p.N, n), fd[a]);
@@ -402,9 +406,10 @@ template <typename S, int QH, bool DO_H> constexpr int step_min_blocks() {
 // register allocation); CUM: the Cumulants-1st h kind; TRT: the CM-TRT kind
 // with its rates fixed at compile time.  WM (wall mode): 0 every node; 1
 // every node but the wall nodes; 2 the wall nodes only, one thread per entry
-// of the wall table (modes 1 and 2 together make one step; see launch_step)
+// of the wall table (modes 1 and 2 together make one step; see launch_step).
+// FI, FO: elements per population of f in fA and fB (2: low halves of words)
 template <typename S, int QH, bool DO_H, bool REC, bool CUM = false, bool EQ = false, bool PRE = false,
-          bool TRT = false, int WM = 0>
+          bool TRT = false, int WM = 0, uint32_t FI = paired<S, QH>() ? 2u : 1u, uint32_t FO = FI>
 __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step(const S* __restrict__ fA, S* __restrict__ fB,
                                                   const S* __restrict__ hA, S* __restrict__ hB,
                                                   const uint8_t* __restrict__ flags,
@@ -434,7 +439,7 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
     if (type == T_INLET) {
         if (p.zou_he) return;  // k_inlet writes these nodes, possibly at this moment
 #pragma unroll
-        for (int a = 0; a < 27; ++a) st(pop<S, QH>(fB, a, N, n), inlet[a]);
+        for (int a = 0; a < 27; ++a) st(fB + FO * soa(a, N, n), inlet[a]);
         if (DO_H || paired<S, QH>()) {
 #pragma unroll
             for (int i = 0; i < QH; ++i) {
@@ -448,7 +453,7 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
             urec[2 * N + n] = par<R>(p.uin[2], p.pf.uin[2]);
         }
         if constexpr (step_fills_symmetry(sizeof(S), QH, DO_H, REC))
-            store_symmetry_rows<S, QH, DO_H>(fB, hB, n, p);
+            store_symmetry_rows<S, QH, DO_H, FO>(fB, hB, n, p);
         return;
     }
     uint32_t mask = 0;
@@ -472,7 +477,7 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
         for (int a = 0; a < 27; ++a) fd[a] = from_bits<R>((S*)nullptr, word[a] & 0xffffu);
     } else {
 #pragma unroll
-        for (int a = 0; a < 27; ++a) fd[a] = ld<R>(fA + soa(a, N, src_of(nb, a)));
+        for (int a = 0; a < 27; ++a) fd[a] = ld<R>(fA + FI * soa(a, N, src_of(nb, a)));
     }
     if (WM == 2) {
         // wall nodes alone, so every lane has links: the link bodies without
@@ -484,8 +489,8 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
             const bool has = (mask >> a) & 1u;
             const float q = has ? __ldg(lq + off + __popc(mask & ((1u << a) - 1u))) : 0.5f;
             const bool thin = (mask >> b) & 1u;
-            const R fa_b = has ? ld<R>(pop<S, QH>(fA, a, N, n)) : R(0);
-            const R fb_b = has ? ld<R>(pop<S, QH>(fA, b, N, n)) : R(0);
+            const R fa_b = has ? ld<R>(fA + FI * soa(a, N, n)) : R(0);
+            const R fb_b = has ? ld<R>(fA + FI * soa(b, N, n)) : R(0);
             const R qq = (R)fmaxf(q, 0.5f);
             const R v_lin = R(2) * (R)q * fa_b + (R(1) - R(2) * (R)q) * fd[a];
             const R v_far = wdiv<R>(fa_b + (R(2) * qq - R(1)) * fb_b, R(2) * qq);
@@ -500,12 +505,12 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
             if (!(mask & (1u << a))) continue;
             const float q = __ldg(lq + off + __popc(mask & ((1u << a) - 1u)));
             const bool thin = (mask >> b) & 1u;  // x_f = x_b - e_a is solid too
-            const R fa_b = ld<R>(pop<S, QH>(fA, a, N, n));
+            const R fa_b = ld<R>(fA + FI * soa(a, N, n));
             if (q <= 0.5f && !thin) {
                 fd[b] = R(2) * (R)q * fa_b + (R(1) - R(2) * (R)q) * fd[a];  // fd[a] = f*_a(x_f)
             } else {
                 const R qq = (R)fmaxf(q, 0.5f);
-                const R fb_b = ld<R>(pop<S, QH>(fA, b, N, n));
+                const R fb_b = ld<R>(fA + FI * soa(b, N, n));
                 fd[b] = wdiv<R>(fa_b + (R(2) * qq - R(1)) * fb_b, R(2) * qq);
             }
         }
@@ -528,7 +533,7 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
         for (int k = 0; k < 10; ++k) ((R*)frec)[soa(k, N, n)] = m[k];
     }
     Rounded27 fc;
-    collide_store_f<S, QH>(fd, fB, n, p, ux, uy, uz, rs, fc);
+    collide_store_f<S, QH, FO>(fd, fB, n, p, ux, uy, uz, rs, fc);
     if constexpr (!DO_H && paired<S, QH>()) store_f_keep_h<S>(fA, fB, fc, n, N);
     if (REC) {
         urec[n] = ux;
@@ -601,7 +606,7 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S, QH, DO_H>()) k_step
     }
     collide_store_h<S, QH, CUM, TRT>(hd, fB, hB, n, p, ux, uy, uz, Q, rs, fc);
     }
-    if constexpr (step_fills_symmetry(sizeof(S), QH, DO_H, REC)) store_symmetry_rows<S, QH, DO_H>(fB, hB, n, p);
+    if constexpr (step_fills_symmetry(sizeof(S), QH, DO_H, REC)) store_symmetry_rows<S, QH, DO_H, FO>(fB, hB, n, p);
 }
 
 // With many wall nodes the plain 16-bit step runs as two launches: every
@@ -684,7 +689,18 @@ cudaError_t launch_step(const Buffers& b, const DevParams& p, cudaStream_t s, bo
             default: k_step<S, QH, true, true, true, true><<<grid, kBlock, 0, s>>>(LBM_STEP_ARGS); break;
         }
     }
-    else if (urec) k_step<S, QH, false, true><<<grid, kBlock, 0, s>>>(LBM_STEP_ARGS);
+    else if (urec) {
+        if constexpr (sizeof(S) == 2 && QH == 7) {
+            if (b.f_words) {  // (a run has two steps or more, so never both)
+                if (b.f_words == 1)
+                    k_step<S, QH, false, true, false, false, false, false, 0, 2, 1><<<grid, kBlock, 0, s>>>(LBM_STEP_ARGS);
+                else
+                    k_step<S, QH, false, true, false, false, false, false, 0, 1, 2><<<grid, kBlock, 0, s>>>(LBM_STEP_ARGS);
+                return cudaGetLastError();
+            }
+        }
+        k_step<S, QH, false, true><<<grid, kBlock, 0, s>>>(LBM_STEP_ARGS);
+    }
     else k_step<S, QH, false, false><<<grid, kBlock, 0, s>>>(LBM_STEP_ARGS);
 #undef LBM_STEP_ARGS
     return cudaGetLastError();
@@ -1589,7 +1605,7 @@ __device__ __forceinline__ void zou_he_fill_h(T* hd, T drho, T ux, T uy, T uz, c
 // frec, hrec: pre-collision records of the coupled adjoint (the f moments and,
 // after them, the inlet node's full arrival vector after the rule; the h
 // arrivals), or nullptr
-template <typename S, int QH, bool CUM, bool DO_H>
+template <typename S, int QH, bool CUM, bool DO_H, uint32_t FI = paired<S, QH>() ? 2u : 1u, uint32_t FO = FI>
 __global__ void __launch_bounds__(kBlock) k_inlet(const S* __restrict__ fA, S* __restrict__ fB,
                                                    const S* __restrict__ hA, S* __restrict__ hB,
                                                    const uint8_t* __restrict__ flags,
@@ -1607,7 +1623,7 @@ __global__ void __launch_bounds__(kBlock) k_inlet(const S* __restrict__ fA, S* _
     const R ux = par<R>(p.uin[0], p.pf.uin[0]), uy = par<R>(p.uin[1], p.pf.uin[1]), uz = par<R>(p.uin[2], p.pf.uin[2]);
     R fd[27];
 #pragma unroll
-    for (int a = 0; a < 27; ++a) fd[a] = (EX(a) == 1) ? R(0) : ld<R>(pop<S, QH>(fA, a, p.N, src_of(nb, a)));
+    for (int a = 0; a < 27; ++a) fd[a] = (EX(a) == 1) ? R(0) : ld<R>(fA + FI * soa(a, p.N, src_of(nb, a)));
     const R drho = zou_he_fill_f<R>(fd, ux, uy, uz, p);
     if (frec) {
         R m[10];
@@ -1621,7 +1637,7 @@ __global__ void __launch_bounds__(kBlock) k_inlet(const S* __restrict__ fA, S* _
     R vx, vy, vz;
     SrStream rs{sr_bits((uint32_t)n, (p.step_ctr ? *p.step_ctr : 0u) + p.step)};
     Rounded27 fc;
-    collide_store_f<S, QH>(fd, fB, n, p, vx, vy, vz, rs, fc);
+    collide_store_f<S, QH, FO>(fd, fB, n, p, vx, vy, vz, rs, fc);
     if constexpr (!DO_H && paired<S, QH>()) store_f_keep_h<S>(fA, fB, fc, n, N);
     if (urec) {
         urec[n] = vx;
@@ -1643,7 +1659,7 @@ __global__ void __launch_bounds__(kBlock) k_inlet(const S* __restrict__ fA, S* _
         const R Q = theta ? (R)__ldg(theta + n) : R(0);
         collide_store_h<S, QH, CUM>(hd, fB, hB, n, p, vx, vy, vz, Q, rs, fc);
     }
-    if constexpr (step_fills_symmetry(sizeof(S), QH, DO_H, false)) store_symmetry_rows<S, QH, DO_H>(fB, hB, n, p);
+    if constexpr (step_fills_symmetry(sizeof(S), QH, DO_H, false)) store_symmetry_rows<S, QH, DO_H, FO>(fB, hB, n, p);
 }
 
 template <typename S, int QH>
@@ -1653,6 +1669,13 @@ cudaError_t launch_inlet(const Buffers& b, const DevParams& p, cudaStream_t s, b
     const int grid = (total + kBlock - 1) / kBlock;
 #define LBM_INLET_ARGS                                                                                   \
     (const S*)b.fA, (S*)b.fB, (const S*)b.hA, (S*)b.hB, b.flags, b.theta, (R*)b.urec, b.frec, b.hrec, p
+    if constexpr (sizeof(S) == 2 && QH == 7) {
+        if (!advance_h && b.f_words) {
+            if (b.f_words == 1) k_inlet<S, QH, false, false, 2, 1><<<grid, kBlock, 0, s>>>(LBM_INLET_ARGS);
+            else k_inlet<S, QH, false, false, 1, 2><<<grid, kBlock, 0, s>>>(LBM_INLET_ARGS);
+            return cudaGetLastError();
+        }
+    }
     if (!advance_h) k_inlet<S, QH, false, false><<<grid, kBlock, 0, s>>>(LBM_INLET_ARGS);
     else if (p.hkind == 3) k_inlet<S, QH, true, true><<<grid, kBlock, 0, s>>>(LBM_INLET_ARGS);
     else k_inlet<S, QH, false, true><<<grid, kBlock, 0, s>>>(LBM_INLET_ARGS);
