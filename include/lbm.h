@@ -237,12 +237,13 @@ lbm_status lbm_state_size(lbm_ctx* ctx, size_t* bytes);
 
 /* Copy the stored populations (with a header naming the grid, lattice and
  * storage) to a buffer of *bytes bytes, host memory or (is_device = 1) device
- * memory; *bytes is set to the size used.  Synchronises. */
+ * memory, also of another GPU; *bytes is set to the size used.  Values at nodes
+ * that are no part of the flow (solid, symmetry rows) mean nothing.  Synchronises. */
 lbm_status lbm_save_state(lbm_ctx* ctx, void* buf, size_t* bytes, int is_device);
 
 /* Restore a state written by lbm_save_state of a context with the same grid,
  * lattice and storage (LBM_ERR_INVALID otherwise); buf in host or
- * (is_device = 1) device memory. */
+ * (is_device = 1) device memory, also of another GPU. */
 lbm_status lbm_load_state(lbm_ctx* ctx, const void* buf, size_t bytes, int is_device);
 
 /* ---- adjoint of the h evolution -------------------------------------------

@@ -2466,7 +2466,7 @@ __device__ __forceinline__ void adjoint_flow_node(
 // per node took 96 B of the f part's 460 B per node, six operations a node on
 // the FP64 pipe, and 1.4 ms to add up at 192x64x64 (60 levels and their
 // recomputation there: 26.30 -> 22.36 ms, with dJ/dQ as WideSum).  Both parts
-// wait on their loads: h 79 us at 80 registers (24 warps per SM), f 61 us at 72
+// wait on their loads: h 79 us at 80 registers (24 warps per SM), f 63 us at 72
 // (28 warps) per level at 192x64x64, where their bytes take 43 and 31 us; 93 and
 // 79 us while the velocity derivatives held a second cube (96 registers).
 template <typename R, int QH, bool CUM, int PART>
